@@ -196,13 +196,21 @@ __global__ void k_set_albedo(const float *alb, int n, float4 *mats, const int32_
     }
 }
 
+// vertices of a triangle record (one row per axis)
+__device__ __forceinline__ void record_vertices(const float4 *T, float3 &v0, float3 &v1, float3 &v2) {
+    v0 = f3(T[0].x, T[1].x, T[2].x);
+    v1 = f3(T[0].y, T[1].y, T[2].y);
+    v2 = f3(T[0].z, T[1].z, T[2].z);
+}
+
 // shading records in leaf order: normal of the winding + light unit, material
 __global__ void k_shading_records(const float4 *tris, const float4 *mats, const int32_t *tri_unit, int n,
                                   float4 *shrec) {
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        const float4 p0 = tris[3 * k], p1 = tris[3 * k + 1], p2 = tris[3 * k + 2];
-        const int orig = __float_as_int(p0.w);
-        const float3 ng = normalize(cross(xyz(p1) - xyz(p0), xyz(p2) - xyz(p0)));
+        float3 v0, v1, v2;
+        record_vertices(tris + 3 * (size_t)k, v0, v1, v2);
+        const int orig = __float_as_int(tris[3 * (size_t)k].w);
+        const float3 ng = normalize(cross(v1 - v0, v2 - v0));
         shrec[2 * (size_t)k] = make_float4(ng.x, ng.y, ng.z, __int_as_float(tri_unit[orig]));
         shrec[2 * (size_t)k + 1] = mats[orig];
     }
@@ -306,7 +314,8 @@ __global__ void k_hidden_guide(const uint32_t *cdf, int n, uint32_t *guide) {
 __global__ void k_hidden_area(const float4 *t4, const int32_t *leaf_of, int first, int n, double *area) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int k = leaf_of[first + i];
-        const float4 a = t4[3 * k], b = t4[3 * k + 1], c = t4[3 * k + 2];
+        float3 a, b, c;
+        record_vertices(t4 + 3 * (size_t)k, a, b, c);
         const float v[9] = {a.x, a.y, a.z, b.x, b.y, b.z, c.x, c.y, c.z};
         area[i] = tri_area_d(v);
     }

@@ -1098,9 +1098,8 @@ __global__ void k_reorder(const float *tris, const int *idx, int n, float4 *out)
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         const int p = idx[k];
         const float *t = tris + 9 * (size_t)p;
-        out[3 * k] = make_float4(t[0], t[1], t[2], __int_as_float(p));
-        out[3 * k + 1] = make_float4(t[3], t[4], t[5], 0.f);
-        out[3 * k + 2] = make_float4(t[6], t[7], t[8], 0.f);
+        for (int a = 0; a < 3; ++a)  // one row per axis
+            out[3 * (size_t)k + a] = make_float4(t[a], t[3 + a], t[6 + a], __int_as_float(p));
     }
 }
 

@@ -91,8 +91,9 @@ __global__ void __launch_bounds__(128) k_render_pol(const DevScene s, const PolP
             if (k < 0) break;
             const float3 x = o + d * th;
             if (!(depth == 1 && (p.flags & MT_UNWARP))) opl += th;
-            const float4 p0 = __ldg(&s.tris[3 * k]), p1 = __ldg(&s.tris[3 * k + 1]), p2 = __ldg(&s.tris[3 * k + 2]);
-            const float3 ng = normalize(cross(xyz(p1) - xyz(p0), xyz(p2) - xyz(p0)));
+            float3 v0, v1, v2;
+            tri_vertices(s, k, v0, v1, v2);
+            const float3 ng = normalize(cross(v1 - v0, v2 - v0));
             const float3 wo = -d;
             const float cwo = dot(ng, wo);
             const int unit = __ldg(&s.tri_unit[orig]);

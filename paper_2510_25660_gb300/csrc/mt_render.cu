@@ -377,8 +377,9 @@ struct Tracer {
         cnt.vertices++;
         const float3 x = ps.o + ps.d * th;
         if (!(ps.depth == 1 && (p.flags & MT_UNWARP))) ps.opl += th;
-        const float4 p0 = ldg_keep(&s.tris[3 * k]), p1 = ldg_keep(&s.tris[3 * k + 1]), p2 = ldg_keep(&s.tris[3 * k + 2]);
-        const float3 ng = normalize(cross(xyz(p1) - xyz(p0), xyz(p2) - xyz(p0)));
+        float3 v0, v1, v2;
+        tri_vertices(s, k, v0, v1, v2);
+        const float3 ng = normalize(cross(v1 - v0, v2 - v0));
         const float3 wo = -ps.d;
         const float cwo = dot(ng, wo);
         const int unit = __ldg(&s.tri_unit[orig]);
