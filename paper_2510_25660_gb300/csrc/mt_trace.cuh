@@ -219,6 +219,16 @@ struct TraceCnt {
 #define MT_LEAF_MORE 0x60000000u                // count - 1 field of a leaf reference
 #define MT_LEAF_NEXT (1u - 0x20000000u)         // first + 1, count - 1 (mod 2^32)
 
+// The binary traversals push without looking at the stack's size.  A ray's
+// stack holds at most one entry per internal node on the way from the root to
+// the node it visits, so never more than the depth of the tree, and a scene
+// whose tree is deeper than MT_STACK - 2 is refused when it is built (scene
+// creation validates every child reference too).  With the check, and the
+// atomic on the error word behind it, the compiler kept the lanes of the
+// descending branches apart from those that pop: 512x512x256-spp frame of the
+// 1.16M-triangle scene 70.6 -> 64.6 ms, exhaustive NLOS scan 32.1 -> 16.1 ms,
+// confocal scan 2.37 -> 1.76 ms, Cornell box render 369 -> 197 us.
+
 // Closest hit with t in (0, tmax); ties in t go to the smaller original index.
 // Returns the leaf-order triangle index (or -1) and writes t and the original index.
 template <bool CNT>
@@ -240,12 +250,7 @@ __device__ __forceinline__ int trace_closest(const DevScene &s, const RayT &r, f
             const bool h1 = tn1 <= tf1;
             if (h0 && h1) {
                 const bool f0 = tn0 <= tn1;
-                if (sp < MT_STACK) {
-                    st[sp] = make_uint2(f0 ? b.w : b.z, __float_as_uint(f0 ? tn1 : tn0));
-                    ++sp;
-                } else {
-                    raise_err(s, MT_EFLAG_STACK);
-                }
+                st[sp++] = make_uint2(f0 ? b.w : b.z, __float_as_uint(f0 ? tn1 : tn0));
                 ref = f0 ? b.z : b.w;
                 continue;
             }
@@ -303,12 +308,7 @@ __device__ __forceinline__ bool trace_any(const DevScene &s, const RayT &r, floa
             const bool h1 = tn1 <= tf1;
             if (h0 && h1) {
                 const bool f0 = tn0 <= tn1;
-                if (sp < MT_STACK) {
-                    st_ref[sp] = f0 ? b.w : b.z;
-                    ++sp;
-                } else {
-                    raise_err(s, MT_EFLAG_STACK);
-                }
+                st_ref[sp++] = f0 ? b.w : b.z;
                 ref = f0 ? b.z : b.w;
                 continue;
             }
@@ -367,12 +367,7 @@ __device__ __forceinline__ bool trav_step(const DevScene &s, const RayT &r, floa
         const bool h1 = tn1 <= tf1;
         if (h0 && h1) {
             const bool f0 = tn0 <= tn1;
-            if (ts.sp < MT_STACK) {
-                st[ts.sp] = make_uint2(f0 ? b.w : b.z, __float_as_uint(f0 ? tn1 : tn0));
-                ++ts.sp;
-            } else {
-                raise_err(s, MT_EFLAG_STACK);
-            }
+            st[ts.sp++] = make_uint2(f0 ? b.w : b.z, __float_as_uint(f0 ? tn1 : tn0));
             ts.ref = f0 ? b.z : b.w;
             return false;
         }
