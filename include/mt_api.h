@@ -330,8 +330,9 @@ mt_status mt_scene_stats(mt_scene scene, int64_t *out);
  *   ctas_per_sm  cap on resident CTAs per SM (0 = occupancy maximum)
  *   priv_bins    time bins per pixel (scan row) accumulated in shared memory
  *                before one write to HBM; later bins are added to the film in
- *                global memory directly.  -1 = as many as fit (default),
- *                0 = none.
+ *                global memory directly.  -1 = as many as fit, 0 = none (of a
+ *                new scene: RENDER, BACKWARD and NLOS_EXHAUSTIVE none, NLOS as
+ *                many as fit).
  *   options      MT_OPT_* bits (below). */
 mt_status mt_set_launch(mt_scene scene, int32_t kind, int32_t threads, int32_t tile, int32_t ctas_per_sm,
                         int32_t priv_bins, uint32_t options);

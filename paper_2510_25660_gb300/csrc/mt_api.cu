@@ -593,6 +593,11 @@ static mt_status scene_create_impl(const float *tris, int64_t n, const mt_materi
     D.err = sc->err;
     D.counters = sc->counters;
     for (int k = 0; k < 4; ++k) sc->cfg[k] = LaunchCfg{256, 0, 0, sc->num_sms, 0, -1, 0};
+    // renders and backward passes add to the film in L2 instead of privatising it: zeroing and writing a
+    // warp's histograms costs more than the few adds of its paths, and the shared memory costs resident
+    // CTAs (97k triangles, 135x241 px, 19 spp: 1150 us against 1628 with all bins that fit; Cornell box
+    // 64x64, 16 spp: 110 against 144 us; backward passes 1291 against 1905 and 176 against 204 us)
+    sc->cfg[MT_LAUNCH_RENDER].priv = sc->cfg[MT_LAUNCH_BACKWARD].priv = 0;
     // exhaustive NLOS grids: 32 sensors per tile with every splat in global memory (measured 130 ms
     // against 190 ms at the automatic 6-row tiles with shared-memory histograms)
     sc->cfg[MT_LAUNCH_NLOS_EXHAUSTIVE] = LaunchCfg{256, 32, 0, sc->num_sms, 0, 0, 0};
@@ -851,15 +856,25 @@ static LaunchCfg render_cfg(const mt_scene_s *s, int kind, int32_t W, int32_t T,
     return c;
 }
 
-// warp-owned tiles of k_render: `tile` pixels per warp (default: enough pixels
-// for 64 paths), D = bins per pixel privatised in the warp's shared-memory
-// slice (priv < 0: as many as fit in ~100 KB per CTA; bins >= D go to global
-// memory with red.add)
-static LaunchCfg warp_tile_cfg(const mt_scene_s *s, int kind, int32_t W, int32_t T, int32_t spp, int extra_floats,
-                               int &D) {
+// warp-owned tiles of k_render: `tile` pixels per warp, D = bins per pixel
+// privatised in the warp's shared-memory slice (priv = -1: as many as fit in
+// ~100 KB per CTA; bins >= D go to global memory with red.add).
+// The automatic tile holds 32 paths, one per lane: more paths in a warp only
+// lengthen its serial chain of traversals.  A frame of fewer than 32 paths for
+// each of 16 warps per SM is spread over that many warps instead (down to one
+// path each): a warp with fewer lanes diverges less and the chip is idle
+// otherwise.  Measured, tiles of 1 / 2 / 4 / 8 pixels without privatisation:
+// Cornell box 23x37 px, 1 spp: 37 / 43 / 48 / 51 us; 64x64, 16 spp: 130 / 110
+// / 189 / 346; 128x128, 1 spp: 155 / 119 / 95 / 78; 97k triangles 135x241, 19
+// spp: 1357 / 1150 / 1242 / 1633 (tiles of 64 paths with all bins that fit: 126,
+// 198, 176 and 2260 us).
+static LaunchCfg warp_tile_cfg(const mt_scene_s *s, int kind, int32_t H, int32_t W, int32_t T, int32_t spp,
+                               int extra_floats, int &D) {
     LaunchCfg c = s->cfg[kind];
     const int warps = c.threads / 32;
-    int tile = c.tile > 0 ? c.tile : std::max(1, (64 + spp - 1) / spp);
+    const long long total = (long long)H * W * spp;
+    const int paths = (int)std::max<long long>(1, std::min<long long>(32, total / (16LL * s->num_sms)));
+    int tile = c.tile > 0 ? c.tile : (int)((paths + (long long)spp - 1) / spp);
     tile = std::max(1, std::min(tile, W));
     const size_t cap = (size_t)std::min(s->smem_optin, 220 * 1024) - 1024;
     const size_t budget = std::min(cap, (size_t)100 * 1024);
@@ -1115,7 +1130,7 @@ static mt_status render_common(mt_scene s, mt_film f, int32_t spp, uint64_t seed
     const int kind = mode == 2 ? MT_LAUNCH_BACKWARD : MT_LAUNCH_RENDER;
     const int n_em_smem = (mode == 2 && s->n_em <= 64) ? s->n_em : 0;
     int D;
-    LaunchCfg cfg = warp_tile_cfg(s, kind, f->W, f->T, spp, n_em_smem * 3, D);
+    LaunchCfg cfg = warp_tile_cfg(s, kind, f->H, f->W, f->T, spp, n_em_smem * 3, D);
     RenderParams p{};
     p.H = f->H;
     p.W = f->W;
