@@ -384,6 +384,21 @@ __global__ void k_max(const float *v, size_t n, unsigned int *out) {
     if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(m));  // non-negative floats order as uints
 }
 
+// the eight corner densities of every cell of the grid (cell (x, y, z) lies between the voxel centres x - 1
+// and x, ..., clamped at the border), one 32-byte record each
+__global__ void k_cells(const float *dens, int rx, int ry, int rz, float4 *cells) {
+    const size_t n = (size_t)(rx + 1) * (ry + 1) * (rz + 1);
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const int x = (int)(i % (rx + 1)), y = (int)(i / (rx + 1) % (ry + 1)),
+                  z = (int)(i / ((size_t)(rx + 1) * (ry + 1)));
+        const int x0 = max(x - 1, 0), x1 = min(x, rx - 1), y0 = max(y - 1, 0), y1 = min(y, ry - 1),
+                  z0 = max(z - 1, 0), z1 = min(z, rz - 1);
+        auto D = [&](int a, int b, int c) { return dens[((size_t)c * ry + b) * rx + a]; };
+        cells[2 * i] = make_float4(D(x0, y0, z0), D(x1, y0, z0), D(x0, y1, z0), D(x1, y1, z0));
+        cells[2 * i + 1] = make_float4(D(x0, y0, z1), D(x1, y0, z1), D(x0, y1, z1), D(x1, y1, z1));
+    }
+}
+
 __global__ void k_probe_philox(uint32_t k0, uint32_t k1, const uint4 *c, long long n, uint4 *o) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         o[i] = philox4x32_10(c[i], k0, k1);
@@ -438,6 +453,13 @@ int grid_for(long long n, int threads, int num_sms) {
 extern "C" {
 
 const char *mt_last_error(void) { return mt::get_error(); }
+
+// Largest array of density-cell records a medium gets.  The records are eight times the grid; this much still
+// stays in L2 (129 MB) beside the path state, and a larger grid, whose records would be gathered from DRAM
+// while the grid itself fits L2, is read voxel by voxel.
+#ifndef MT_CELL_BYTES
+#define MT_CELL_BYTES (96ull << 20)
+#endif
 
 static mt_status scene_create_impl(const float *tris, int64_t n, const mt_material *mats, const mt_emitter *ems,
                                    int32_t n_em, const mt_camera *cam, const mt_medium *med, cudaStream_t st,
@@ -567,6 +589,14 @@ static mt_status scene_create_impl(const float *tris, int64_t n, const mt_materi
         D.rz = med->res[2];
         D.m_lo = make_float3(med->lo[0], med->lo[1], med->lo[2]);
         D.m_hi = make_float3(med->hi[0], med->hi[1], med->hi[2]);
+        D.m_ext = make_float3(med->hi[0] - med->lo[0], med->hi[1] - med->lo[1], med->hi[2] - med->lo[2]);
+        D.m_rext = make_float3(1.0f / D.m_ext.x, 1.0f / D.m_ext.y, 1.0f / D.m_ext.z);
+        const uint64_t n_cells = (uint64_t)(D.rx + 1) * (D.ry + 1) * (D.rz + 1);
+        float4 *cells = nullptr;  // a scene that has no room for them reads the grid
+        if (n_cells * 32 <= MT_CELL_BYTES && al.alloc(&cells, 2 * (size_t)n_cells, "density cells") == MT_OK) {
+            k_cells<<<grid_for((long long)n_cells, 256, sc->num_sms), 256, 0, st>>>(dens, D.rx, D.ry, D.rz, cells);
+            D.cells = reinterpret_cast<const float *>(cells);
+        }
     }
     // scratch
     MT_TRY(al.alloc(&sc->tile_counter, 4, "tile counters"));

@@ -287,8 +287,10 @@ struct DevScene {
     float3 q_lo, q_scale;  // BVH plane quantisation: plane = q_lo + q * q_scale
     // medium
     const float *dens;     // [z][y][x]
+    const float *cells;    // the 8 corner densities of every cell, [rz + 1][ry + 1][rx + 1][8] (null: large grids)
     int32_t rx, ry, rz;
     float3 m_lo, m_hi;
+    float3 m_ext, m_rext;  // m_hi - m_lo and its reciprocal, each rounded to nearest
     float m_major;
     const float *m_params; // device [2]: albedo, g
     uint32_t *err;
@@ -300,21 +302,45 @@ __device__ __forceinline__ void raise_err(const DevScene &s, uint32_t bit) { ato
 // ---------------------------------------------------------------------------
 // participating medium (Sec. 4.1): trilinear density, box overlap, ratio tracking
 // ---------------------------------------------------------------------------
+// a / c rounded to nearest, given rc = 1 / c rounded to nearest: a * rc corrected by its exact FMA remainder
+// (Markstein, IBM J. Res. Dev. 34, 1990; Brisebarre, Muller and Raina, IEEE Trans. Computers 53, 2004, for a
+// divisor known in advance).  a and a / c in the normal range.
+__device__ __forceinline__ float div_known(float a, float c, float rc) {
+    const float q = a * rc;
+    return fmaf(fmaf(-q, c, a), rc, q);
+}
+
+// Trilinear density at p.  The tracking loops are bound by instruction issue at a few lanes per instruction
+// (a warp walks as long as its longest ray), so the lookup is kept short: grids whose cell records fit take the
+// eight corners of the cell in one 32-byte load instead of eight loads of their own addresses (media training
+// step 79.2 -> 73.2 ms for a 128^3 grid), and the coordinates divide by the box extents without a divide's
+// slow-path branch (73.1 -> 70.6 ms).
 __device__ __forceinline__ float density_at(const DevScene &s, float3 p) {
-    const float gx = (p.x - s.m_lo.x) / (s.m_hi.x - s.m_lo.x) * s.rx - 0.5f;
-    const float gy = (p.y - s.m_lo.y) / (s.m_hi.y - s.m_lo.y) * s.ry - 0.5f;
-    const float gz = (p.z - s.m_lo.z) / (s.m_hi.z - s.m_lo.z) * s.rz - 0.5f;
+    const float gx = div_known(p.x - s.m_lo.x, s.m_ext.x, s.m_rext.x) * s.rx - 0.5f;
+    const float gy = div_known(p.y - s.m_lo.y, s.m_ext.y, s.m_rext.y) * s.ry - 0.5f;
+    const float gz = div_known(p.z - s.m_lo.z, s.m_ext.z, s.m_rext.z) * s.rz - 0.5f;
     const float fx0 = floorf(gx), fy0 = floorf(gy), fz0 = floorf(gz);
     const float fx = gx - fx0, fy = gy - fy0, fz = gz - fz0;
     const int ix = (int)fx0, iy = (int)fy0, iz = (int)fz0;
-    const int x0 = min(max(ix, 0), s.rx - 1), x1 = min(max(ix + 1, 0), s.rx - 1);
-    const int y0 = min(max(iy, 0), s.ry - 1), y1 = min(max(iy + 1, 0), s.ry - 1);
-    const int z0 = min(max(iz, 0), s.rz - 1), z1 = min(max(iz + 1, 0), s.rz - 1);
-    auto D = [&](int x, int y, int z) { return __ldg(&s.dens[((size_t)z * s.ry + y) * s.rx + x]); };
-    const float c00 = D(x0, y0, z0) * (1.f - fx) + D(x1, y0, z0) * fx;
-    const float c10 = D(x0, y1, z0) * (1.f - fx) + D(x1, y1, z0) * fx;
-    const float c01 = D(x0, y0, z1) * (1.f - fx) + D(x1, y0, z1) * fx;
-    const float c11 = D(x0, y1, z1) * (1.f - fx) + D(x1, y1, z1) * fx;
+    float v[8];  // corners, x fastest
+    if (s.cells) {
+        const int cx = min(max(ix + 1, 0), s.rx), cy = min(max(iy + 1, 0), s.ry), cz = min(max(iz + 1, 0), s.rz);
+        const float *c = s.cells + 8 * (size_t)(uint32_t)((cz * (s.ry + 1) + cy) * (s.rx + 1) + cx);
+        asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+            : "l"(c));
+    } else {
+        const int x0 = min(max(ix, 0), s.rx - 1), x1 = min(max(ix + 1, 0), s.rx - 1);
+        const int y0 = min(max(iy, 0), s.ry - 1), y1 = min(max(iy + 1, 0), s.ry - 1);
+        const int z0 = min(max(iz, 0), s.rz - 1), z1 = min(max(iz + 1, 0), s.rz - 1);
+        auto D = [&](int x, int y, int z) { return __ldg(&s.dens[((size_t)z * s.ry + y) * s.rx + x]); };
+        v[0] = D(x0, y0, z0), v[1] = D(x1, y0, z0), v[2] = D(x0, y1, z0), v[3] = D(x1, y1, z0);
+        v[4] = D(x0, y0, z1), v[5] = D(x1, y0, z1), v[6] = D(x0, y1, z1), v[7] = D(x1, y1, z1);
+    }
+    const float c00 = v[0] * (1.f - fx) + v[1] * fx;
+    const float c10 = v[2] * (1.f - fx) + v[3] * fx;
+    const float c01 = v[4] * (1.f - fx) + v[5] * fx;
+    const float c11 = v[6] * (1.f - fx) + v[7] * fx;
     const float c0 = c00 * (1.f - fy) + c10 * fy, c1 = c01 * (1.f - fy) + c11 * fy;
     return c0 * (1.f - fz) + c1 * fz;
 }
@@ -353,17 +379,14 @@ __device__ __forceinline__ float transmittance(const DevScene &s, const Rng &rng
     if (!medium_span(s, o, d, dist, a, b)) return 1.0f;
     float T = 1.0f, t = a;
     const float inv = 1.0f / s.m_major;
-    for (uint32_t j = 0;; ++j) {
-        if (j >= MT_TRACK_STEPS) {
-            ok = false;
-            return 0.f;
-        }
+    for (uint32_t j = 0; j < MT_TRACK_STEPS; ++j) {
         const uint4 R = rng.raw(pix, smp, depth, G_RATIO + j);
         t += -logf(1.0f - u24(R.x)) * inv;
-        if (t >= b) break;
+        if (t >= b) return T;
         T *= 1.0f - density_at(s, o + d * t) * inv;
     }
-    return T;
+    ok = false;
+    return 0.f;
 }
 
 // exponential draw of mean `mean` from one Philox word (1 - u > 0)

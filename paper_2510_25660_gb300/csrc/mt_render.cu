@@ -332,20 +332,23 @@ struct Tracer {
             const float tsurf = k >= 0 ? th : 1e30f;
             if (medium_span(s, ps.o, ps.d, tsurf, ma, mb)) {
                 float t = ma;
-                bool collided = false;
+                bool collided = false, ended = false;
                 const float inv = 1.0f / s.m_major;
-                for (uint32_t j = 0;; ++j) {
-                    if (j >= MT_TRACK_STEPS) {
-                        raise_err(s, MT_EFLAG_TRACK);
-                        return false;
-                    }
+                for (uint32_t j = 0; j < MT_TRACK_STEPS; ++j) {
                     const uint4 R = rng.raw(gp(ps), ps.smp, (uint32_t)(ps.depth - 1), G_TRACK + j);
                     t += -logf(1.0f - u24(R.x)) * inv;
-                    if (t >= mb) break;
-                    if (u24(R.y) < density_at(s, ps.o + ps.d * t) * inv) {
-                        collided = true;
+                    if (t >= mb) {
+                        ended = true;
                         break;
                     }
+                    if (u24(R.y) < density_at(s, ps.o + ps.d * t) * inv) {
+                        collided = ended = true;
+                        break;
+                    }
+                }
+                if (!ended) {
+                    raise_err(s, MT_EFLAG_TRACK);
+                    return false;
                 }
                 if (collided) {
                     cnt.vertices++;

@@ -355,6 +355,10 @@ __global__ void __launch_bounds__(256) k_wf_generate(const DevScene s, const WfP
 #ifndef MT_WF_TRACE_MINB
 #define MT_WF_TRACE_MINB 6
 #endif
+// in a medium the tracking loops need more registers: media training step 72.6 ms at 6, 70.5 at 5, 70.6 at 4
+#ifndef MT_WF_MEDIA_MINB
+#define MT_WF_MEDIA_MINB 5
+#endif
 
 // hit record: (leaf-order triangle or -1, original triangle, t bits, 1 if the
 // path scatters in the medium at t before reaching that surface)
@@ -398,20 +402,24 @@ __device__ __forceinline__ void ext_rays(const DevScene &s, const WfParams &p, c
                     const uint4 m = p.qmode ? p.ps_m[i] : p.meta[slot];
                     const float inv = 1.0f / s.m_major;
                     float tt = ma;
-                    for (uint32_t j = 0;; ++j) {
-                        if (j >= MT_TRACK_STEPS) {
-                            raise_err(s, MT_EFLAG_TRACK);
-                            k = -1;  // the path is dropped
-                            break;
-                        }
+                    bool ended = false;
+                    for (uint32_t j = 0; j < MT_TRACK_STEPS; ++j) {
                         const uint4 R = philox4x32_10(make_uint4(m.x, m.y, m.z - 1u, G_TRACK + j), p.k0, p.k1);
                         tt += -logf(1.0f - u24(R.x)) * inv;
-                        if (tt >= mb) break;
+                        if (tt >= mb) {
+                            ended = true;
+                            break;
+                        }
                         if (u24(R.y) < density_at(s, xyz(o) + xyz(d) * tt) * inv) {
                             collided = 1;
                             t = tt;
+                            ended = true;
                             break;
                         }
+                    }
+                    if (!ended) {
+                        raise_err(s, MT_EFLAG_TRACK);
+                        k = -1;  // the path is dropped
                     }
                 }
             }
@@ -423,7 +431,8 @@ __device__ __forceinline__ void ext_rays(const DevScene &s, const WfParams &p, c
 }
 
 template <bool WIDE, bool CNT, bool MEDIA>
-__global__ void __launch_bounds__(256, MT_WF_TRACE_MINB) k_wf_extend(const DevScene s, const WfParams p, const uint32_t *qcur) {
+__global__ void __launch_bounds__(256, MEDIA ? MT_WF_MEDIA_MINB : MT_WF_TRACE_MINB)
+    k_wf_extend(const DevScene s, const WfParams p, const uint32_t *qcur) {
     TraceCnt tc{0, 0};
     uint32_t rays = 0;
     ext_rays<WIDE, CNT, MEDIA>(s, p, qcur, tc, rays);
@@ -1287,7 +1296,8 @@ __device__ __forceinline__ void sh_rays(const DevScene &s, const WfParams &p, ui
 
 // shadow rays of this iteration's shading; n_idx names the counter that holds their number
 template <bool DUMP, bool CNT, bool WIDE, bool MEDIA, bool BWD>
-__global__ void __launch_bounds__(256, MT_WF_TRACE_MINB) k_wf_shadow(const DevScene s, const WfParams p, int n_idx) {
+__global__ void __launch_bounds__(256, MEDIA ? MT_WF_MEDIA_MINB : MT_WF_TRACE_MINB)
+    k_wf_shadow(const DevScene s, const WfParams p, int n_idx) {
     __shared__ float em_acc[BWD ? MT_WF_EM_SMEM * 3 : 1];
     if (BWD) {
         for (int k = threadIdx.x; k < MT_WF_EM_SMEM * 3; k += blockDim.x) em_acc[k] = 0.f;
@@ -1310,7 +1320,8 @@ __global__ void __launch_bounds__(256, MT_WF_TRACE_MINB) k_wf_shadow(const DevSc
 // each other), so that warps that find the extension queue drained trace
 // shadow rays instead of idling in the tail of the pass.
 template <bool WIDE, bool CNT, bool MEDIA, bool DUMP>
-__global__ void __launch_bounds__(256, MT_WF_TRACE_MINB) k_wf_trace(const DevScene s, const WfParams p, const uint32_t *qcur) {
+__global__ void __launch_bounds__(256, MEDIA ? MT_WF_MEDIA_MINB : MT_WF_TRACE_MINB)
+    k_wf_trace(const DevScene s, const WfParams p, const uint32_t *qcur) {
     TraceCnt tc{0, 0};
     uint32_t rays = 0, contribs = 0;
     ext_rays<WIDE, CNT, MEDIA>(s, p, qcur, tc, rays);
