@@ -322,17 +322,18 @@ mt_status mt_scene_stats(mt_scene scene, int64_t *out);
  * autotuner; 0 keeps a field at its default), per kind: MT_LAUNCH_RENDER,
  * MT_LAUNCH_BACKWARD, MT_LAUNCH_NLOS (scan-point grids) and
  * MT_LAUNCH_NLOS_EXHAUSTIVE (laser x sensor grids, whose scene default is 32
- * sensors per tile with priv_bins = 0: the lanes of a warp take consecutive
+ * sensors per tile with priv_bins = 0: the lanes of a warp take neighbouring
  * sensors and one hidden sample):
  *   threads      threads per CTA (32..256, multiple of 32)
  *   tile         RENDER/BACKWARD: pixels of one image row owned by one warp at
- *                a time; NLOS: scan rows owned by one CTA at a time
+ *                a time (default: pixels for 32 paths, fewer where the frame
+ *                would not fill the GPU); NLOS: scan rows owned by one CTA at
+ *                a time (default: 1; EXHAUSTIVE 32)
  *   ctas_per_sm  cap on resident CTAs per SM (0 = occupancy maximum)
  *   priv_bins    time bins per pixel (scan row) accumulated in shared memory
  *                before one write to HBM; later bins are added to the film in
- *                global memory directly.  -1 = as many as fit, 0 = none (of a
- *                new scene: RENDER, BACKWARD and NLOS_EXHAUSTIVE none, NLOS as
- *                many as fit).
+ *                global memory directly.  -1 = as many as fit, 0 = none (what
+ *                a new scene uses).
  *   options      MT_OPT_* bits (below). */
 mt_status mt_set_launch(mt_scene scene, int32_t kind, int32_t threads, int32_t tile, int32_t ctas_per_sm,
                         int32_t priv_bins, uint32_t options);

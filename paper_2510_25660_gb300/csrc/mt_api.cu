@@ -120,6 +120,8 @@ struct mt_scene_s {
     float4 *ysamp = nullptr;
     int32_t *ysamp_tri = nullptr;
     long long ysamp_cap = 0;
+    int32_t *sorder = nullptr;  // sensor order of exhaustive grids
+    int32_t sorder_cap = 0;
     GraphCache nlos_graph;
     cudaStream_t cap_stream = nullptr;  // private stream the NLOS graph is captured on
     // wavefront path pool
@@ -628,6 +630,7 @@ static mt_status scene_create_impl(const float *tris, int64_t n, const mt_materi
     // CTAs (97k triangles, 135x241 px, 19 spp: 1150 us against 1628 with all bins that fit; Cornell box
     // 64x64, 16 spp: 110 against 144 us; backward passes 1291 against 1905 and 176 against 204 us)
     sc->cfg[MT_LAUNCH_RENDER].priv = sc->cfg[MT_LAUNCH_BACKWARD].priv = 0;
+    sc->cfg[MT_LAUNCH_NLOS].priv = 0;  // 64x64 points, T = 4096, 1024 samples: 1.51 ms against 1.60 privatised
     // exhaustive NLOS grids: 32 sensors per tile with every splat in global memory (measured 130 ms
     // against 190 ms at the automatic 6-row tiles with shared-memory histograms)
     sc->cfg[MT_LAUNCH_NLOS_EXHAUSTIVE] = LaunchCfg{256, 32, 0, sc->num_sms, 0, 0, 0};
@@ -865,24 +868,21 @@ static void seed_key(uint64_t seed, uint32_t &k0, uint32_t &k1) {
     k1 = (uint32_t)(seed >> 32);
 }
 
-// pick tile size and privatisation depth for a film within the shared-memory budget
-static LaunchCfg render_cfg(const mt_scene_s *s, int kind, int32_t W, int32_t T, int C, int extra_floats, int &D) {
+// tile size and privatisation depth of an NLOS capture within the shared-memory budget
+static LaunchCfg nlos_cfg(const mt_scene_s *s, int kind, int32_t T, int &D) {
     LaunchCfg c = s->cfg[kind];
     const size_t budget = (size_t)std::min(s->smem_optin, 220 * 1024) - 1024;
     int tile = c.tile > 0 ? c.tile : 0;
-    if (tile == 0) {
-        // default: aim for >= 48 KB histograms, up to 32 pixels
-        const size_t per_px = (size_t)T * C * 4;
-        tile = (int)std::max<size_t>(1, std::min<size_t>(32, (96 * 1024) / std::max<size_t>(per_px, 1)));
-        if (kind == MT_LAUNCH_RENDER || kind == MT_LAUNCH_BACKWARD) tile = std::min(tile, W);
-    }
-    size_t fixed = ((size_t)tile * (C == 3 ? 3 : 1) + extra_floats) * 4 + 64;
-    size_t avail = budget > fixed ? budget - fixed : 0;
-    D = (int)std::min<size_t>((size_t)T, avail / ((size_t)tile * C * 4));
+    // automatic: one scan row per CTA (64x64 points, T = 4096, 1024 samples: 1.60 ms with its bins in shared memory,
+    // 1.77 / 2.51 ms for 2 / 4 rows), 32 sensors of a laser
+    if (tile == 0) tile = kind == MT_LAUNCH_NLOS_EXHAUSTIVE ? 32 : 1;
+    const size_t fixed = (size_t)tile * 4 + 64;
+    const size_t avail = budget > fixed ? budget - fixed : 0;
+    D = (int)std::min<size_t>((size_t)T, avail / ((size_t)tile * 4));
     if (c.priv >= 0) D = std::min(D, c.priv);
     if (D < 1) D = 0;
     c.tile = tile;
-    c.smem_bytes = (((size_t)tile * D * C + (size_t)tile * (C == 3 ? 3 : 1) + extra_floats) * 4 + 15) & ~(size_t)15;
+    c.smem_bytes = (((size_t)tile * D + (size_t)tile) * 4 + 15) & ~(size_t)15;
     return c;
 }
 
@@ -1407,8 +1407,8 @@ static void nlos_fill(mt_scene s, mt_film f, const mt_scan *sc, int32_t spp, uin
                       int32_t *ysamp_tri, int *tile_counter, NlosParams &p, LaunchCfg &cfg) {
     const long long rows = sc->mode == MT_EXHAUSTIVE ? (long long)sc->n_lasers * sc->n_sensors : sc->n_lasers;
     int D;
-    cfg = render_cfg(s, sc->mode == MT_EXHAUSTIVE ? MT_LAUNCH_NLOS_EXHAUSTIVE : MT_LAUNCH_NLOS, (int)rows, f->T, 1, 0,
-                     D);
+    const bool exh = sc->mode == MT_EXHAUSTIVE;
+    cfg = nlos_cfg(s, exh ? MT_LAUNCH_NLOS_EXHAUSTIVE : MT_LAUNCH_NLOS, f->T, D);
     p = NlosParams{};
     p.T = f->T;
     p.D = D;
@@ -1442,6 +1442,21 @@ static void nlos_fill(mt_scene s, mt_film f, const mt_scan *sc, int32_t spp, uin
     p.ysamp_tri = ysamp_tri;
     p.tile_counter = tile_counter;
     p.aggregate = (cfg.options & MT_OPT_AGGREGATE) ? 1 : 0;
+    // the default forms add every connection in L2
+    const bool plain = D == 0 && !p.aggregate && cfg.tile == (exh ? 32 : 1);
+    p.scan = plain && !exh && spp >= MT_NLOS_ORDER_SPP && rows * spp >= MT_NLOS_ORDER_TOTAL ? 1 : 0;
+    // runs of 128 hidden samples, shorter (down to 4) where that gives fewer than 64 warps per SM
+    p.run = 0;
+    if (plain && exh) {
+        const long long groups = (long long)sc->n_lasers * ((sc->n_sensors + 31) / 32);
+        p.run = (int)std::max<long long>(4, std::min<long long>(128, groups * spp / (64LL * s->num_sms)));
+        // the item count must fit the claim counter
+        while (groups * ((spp + (long long)p.run - 1) / p.run) > 0x40000000LL && p.run < spp) p.run *= 2;
+        if (groups > 0x40000000LL) p.run = 0;
+    }
+    // a CTA has no more threads than its tile has samples
+    const long long work = (long long)cfg.tile * spp;
+    if (!exh && work < cfg.threads) cfg.threads = std::max(32, (int)((work + 31) / 32 * 32));
 }
 
 static mt_status nlos_prepare(mt_scene s, mt_film f, const mt_scan *sc, int32_t spp, uint64_t seed,
@@ -1485,16 +1500,37 @@ static mt_status nlos_prepare(mt_scene s, mt_film f, const mt_scan *sc, int32_t 
     }
     nlos_fill(s, f, sc, spp, seed, sample_offset, s->hcdf, s->hguide, s->h_area, nullptr, s->ysamp, s->ysamp_tri,
               s->tile_counter + 1, p, cfg);
+    if (p.run && sc->n_sensors > 32 &&
+        (long long)sc->n_lasers * sc->n_sensors * (long long)spp >= MT_NLOS_ORDER_PAIRS) {
+        if (sc->n_sensors > s->sorder_cap) {  // while capturing, or without memory for it: the sensors as given
+            cudaStreamCaptureStatus cs;
+            MT_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
+            int32_t *order = nullptr;
+            if (cs == cudaStreamCaptureStatusNone &&
+                s->al.alloc(&order, (size_t)sc->n_sensors, "nlos sensor order") == MT_OK) {
+                s->sorder = order;
+                s->sorder_cap = sc->n_sensors;
+            }
+        }
+        if (sc->n_sensors <= s->sorder_cap) p.order = s->sorder;
+    }
     return MT_OK;
+}
+
+// kernels of one capture
+static int nlos_launches(const NlosParams &p, bool dump) {
+    return p.mode != MT_EXHAUSTIVE ? 1 : (p.order && !dump ? 3 : 2);
 }
 
 static mt_status nlos_enqueue(mt_scene s, mt_film f, const NlosParams &p, const LaunchCfg &cfg, bool dump,
                               cudaStream_t st) {
     if (p.D < p.T && !(p.flags & MT_ACCUMULATE))
         MT_CUDA_TRY(cudaMemsetAsync(p.film, 0, (size_t)f->H * f->W * f->T * sizeof(float), st));
+    if (p.run && !dump && p.steady && !(p.flags & MT_ACCUMULATE))  // its rows are added to by several warps
+        MT_CUDA_TRY(cudaMemsetAsync(p.steady, 0, (size_t)f->H * f->W * sizeof(float), st));
     if (dump) MT_CUDA_TRY(cudaMemsetAsync(p.dump_count, 0, sizeof(int64_t), st));
     MT_CUDA_TRY(cudaMemsetAsync(p.tile_counter, 0, sizeof(int), st));
-    s->launches += p.mode == MT_EXHAUSTIVE ? 2 : 1;
+    s->launches += nlos_launches(p, dump);
     return mt_launch_nlos(s->dev, p, cfg, dump, (f->flags & MT_COUNTERS) != 0, st);
 }
 
@@ -1536,7 +1572,7 @@ mt_status mt_render_nlos(mt_scene s, mt_film f, const mt_scan *scan, int32_t spp
         gc.key = key;
     }
     MT_CUDA_TRY(cudaGraphLaunch(gc.exec, st));
-    s->launches += scan->mode == MT_EXHAUSTIVE ? 2 : 1;
+    s->launches += nlos_launches(p, false);
     return MT_OK;
 }
 
