@@ -71,6 +71,31 @@ __device__ __forceinline__ uint32_t wf_append(uint32_t *count, bool want) {
     return base + __popc(mask & ((1u << lane) - 1u));
 }
 
+// The appends of a shading step to up to three queues at once (every lane of the warp calls this together): the lanes'
+// slots in queue k in at[k] where want[k].  Lanes 0, 1 and 2 claim the three ranges with one atomic instruction, so
+// the warp waits for one round trip to L2 instead of one per queue (512x512x256-spp render of the 1.16M-triangle scene
+// 64.3 -> 62.8 ms, training steps on the 97k-triangle scene 9.86 -> 9.51 and in a medium 70.4 -> 68.2 ms).
+template <int N>
+__device__ __forceinline__ void wf_append_n(uint32_t *const (&count)[N], const bool (&want)[N], uint32_t (&at)[N]) {
+    const int lane = threadIdx.x & 31;
+    unsigned mask[N];
+    uint32_t *c = count[0];
+    uint32_t m = 0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        mask[k] = __ballot_sync(0xffffffffu, want[k]);
+        if (lane == k) {
+            c = count[k];
+            m = (uint32_t)__popc(mask[k]);
+        }
+    }
+    uint32_t base = 0;
+    if (lane < N && m) base = atomicAdd(c, m);
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        at[k] = __shfl_sync(0xffffffffu, base, k) + __popc(mask[k] & ((1u << lane) - 1u));
+}
+
 // 256-bit global loads and stores (sm_100-class) for the 32-byte halves of a
 // path record, (o, d) and (beta, meta), when the pool is a record per slot, per
 // use: generation stores, extension-ray loads, shading loads, shading stores.
@@ -121,19 +146,36 @@ __device__ __forceinline__ uint4 f4u(float4 v) {
     return make_uint4(__float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z), __float_as_uint(v.w));
 }
 
+// Adds of 4 (2) consecutive floats of the film in one reduction (sm_90 and later); a must be 16 (8) bytes aligned.
+__device__ __forceinline__ void red_add4(float *a, float x, float y, float z, float w) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(a), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
+__device__ __forceinline__ void red_add2(float *a, float x, float y) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(a), "f"(x), "f"(y) : "memory");
+}
+
 // frequency space (Sec. 4.3, Eq. 12): C exp(-i 2 pi opl / lambda); "bin" 2q real, 2q + 1 imaginary.
 // Out of line so that its registers do not weigh on the time-binned path.  lp = film pixel.
+// A wavelength's six floats go as three pairs, which its offset of 24 bytes keeps 8 bytes aligned (512x512x256-spp
+// film of four wavelengths 71.2 -> 66.8 ms).
 __device__ __noinline__ void wf_splat_phasor(const WfParams &p, uint32_t lp, float opl, float3 c) {
-    for (int q = 0; q < p.K; ++q) {
+    float *h = p.film + (size_t)lp * p.T * 3;
+    const bool pairs = ((uintptr_t)p.film & 7) == 0;
+    for (int q = 0; q < p.K; ++q, h += 6) {
         float sn, cs;
         sincospif(2.0f * opl / __ldg(&p.lambdas[q]), &sn, &cs);
-        float *h = p.film + ((size_t)lp * p.T + 2 * q) * 3;
-        red_add_stream(h, c.x * cs);
-        red_add_stream(h + 1, c.y * cs);
-        red_add_stream(h + 2, c.z * cs);
-        red_add_stream(h + 3, -c.x * sn);
-        red_add_stream(h + 4, -c.y * sn);
-        red_add_stream(h + 5, -c.z * sn);
+        if (pairs) {
+            red_add2(h, c.x * cs, c.y * cs);
+            red_add2(h + 2, c.z * cs, -c.x * sn);
+            red_add2(h + 4, -c.y * sn, -c.z * sn);
+        } else {
+            red_add_stream(h, c.x * cs);
+            red_add_stream(h + 1, c.y * cs);
+            red_add_stream(h + 2, c.z * cs);
+            red_add_stream(h + 3, -c.x * sn);
+            red_add_stream(h + 4, -c.y * sn);
+            red_add_stream(h + 5, -c.z * sn);
+        }
     }
 }
 
@@ -499,44 +541,31 @@ __global__ void k_wf_sort_keys(const DevScene s, const WfParams p, const uint32_
 // Shade adds emission Stokes vectors and queues next-event rays with their
 // Stokes contributions; the shadow stage splats those that are unoccluded.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void wf_splat_stokes(const WfParams &p, uint32_t pix, float opl, const float S[3][4]) {
-    const uint32_t lp = pix - p.pix_base;
-    const float x = (opl - p.start) / p.width;
-    const bool in = x >= 0.f && x < (float)p.T;
-    float *f = in ? p.film + ((size_t)lp * p.T + (int)x) * 12 : nullptr;
-    float *st = p.steady + (size_t)lp * 12;
+// One film bin (12 floats, 48 bytes) takes three 16-byte reductions where the film is 16 bytes aligned.
+__device__ __forceinline__ void add_stokes(float *f, bool quads, const float S[3][4]) {
+    if (quads) {
+        red_add4(f, S[0][0], S[1][0], S[2][0], S[0][1]);
+        // the rest is zero for light that met no conductor
+        if (S[0][1] != 0.f || S[1][1] != 0.f || S[2][1] != 0.f || S[0][2] != 0.f || S[1][2] != 0.f || S[2][2] != 0.f ||
+            S[0][3] != 0.f || S[1][3] != 0.f || S[2][3] != 0.f) {
+            red_add4(f + 4, S[1][1], S[2][1], S[0][2], S[1][2]);
+            red_add4(f + 8, S[2][2], S[0][3], S[1][3], S[2][3]);
+        }
+        return;
+    }
 #pragma unroll
     for (int k = 0; k < 4; ++k)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float v = S[c][k];
-            if (v != 0.f) {
-                if (in) atomicAdd(f + k * 3 + c, v);
-                atomicAdd(st + k * 3 + c, v);
-            }
-        }
+        for (int c = 0; c < 3; ++c)
+            if (S[c][k] != 0.f) atomicAdd(f + k * 3 + c, S[c][k]);
 }
 
-__device__ __forceinline__ void load_mueller(const WfParams &p, uint32_t slot, Mueller &P) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const float4 v = p.mueller[(size_t)slot * 12 + c * 4 + r];
-            P.m[c][4 * r] = v.x;
-            P.m[c][4 * r + 1] = v.y;
-            P.m[c][4 * r + 2] = v.z;
-            P.m[c][4 * r + 3] = v.w;
-        }
-}
-
-__device__ __forceinline__ void store_mueller(const WfParams &p, uint32_t slot, const Mueller &P) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-            p.mueller[(size_t)slot * 12 + c * 4 + r] =
-                make_float4(P.m[c][4 * r], P.m[c][4 * r + 1], P.m[c][4 * r + 2], P.m[c][4 * r + 3]);
+__device__ __forceinline__ void wf_splat_stokes(const WfParams &p, uint32_t pix, float opl, const float S[3][4]) {
+    const uint32_t lp = pix - p.pix_base;
+    const float x = (opl - p.start) / p.width;
+    const bool quads = (((uintptr_t)p.film | (uintptr_t)p.steady) & 15) == 0;
+    if (x >= 0.f && x < (float)p.T) add_stokes(p.film + ((size_t)lp * p.T + (int)x) * 12, quads, S);
+    add_stokes(p.steady + (size_t)lp * 12, quads, S);
 }
 
 // GGX microfacet factor D G2 / (4 cos_o cos_i) and the cosine of the microfacet
@@ -551,8 +580,22 @@ __device__ __forceinline__ float ggx_factor(float rough, float3 wol, float3 wil,
     return D * G2 / (4.0f * wol.z * wil.z);
 }
 
-__global__ void __launch_bounds__(128) k_wf_shade_pol(const DevScene s, const WfParams p, const uint32_t *qcur,
-                                                     uint32_t *qnext) {
+// The Mueller throughput of a path (per colour the 4x4 matrix that takes light at its vertex to the sensor) is kept in
+// the form its last vertex left it in (meta.w): the identity of a camera ray (not stored), one column after a
+// Lambertian vertex (an ideal depolariser zeroes the other three; 3 float4 instead of 12, and the frame no longer
+// matters), or the full matrix.  The vertex is sampled first and the colours go through it one after the other, so 16
+// matrix elements are live instead of 48.
+#define MT_POL_IDENTITY 0u
+#define MT_POL_COLUMN 1u
+#define MT_POL_FULL 2u
+// The loop over the colours stays a loop: unrolled, the stage lost three issue slots in each four to instruction
+// fetches.  512x512x64-spp Stokes render of the 1.16M-triangle scene: 26.9 ms with the whole matrix in registers (133
+// of them), 25.0 in this form, 23.4 with the loop kept and eight CTAs per SM (24.1 / 23.8 at four / five).
+#ifndef MT_WF_SHADE_POL_MINB
+#define MT_WF_SHADE_POL_MINB 8
+#endif
+__global__ void __launch_bounds__(128, MT_WF_SHADE_POL_MINB) k_wf_shade_pol(const DevScene s, const WfParams p,
+                                                                            const uint32_t *qcur, uint32_t *qnext) {
     const uint32_t n = p.counters[C_CUR];
     uint32_t verts = 0, contribs = 0;
     const uint32_t stride = gridDim.x * blockDim.x;
@@ -567,7 +610,7 @@ __global__ void __launch_bounds__(128) k_wf_shade_pol(const DevScene s, const Wf
             const float4 o4 = p.o[slot], d4 = p.d[slot];
             const uint4 m = p.meta[slot];
             const int4 h = p.hit[slot];
-            const uint32_t pix = m.x, smp = m.y;
+            const uint32_t pix = m.x, smp = m.y, form = m.w;
             const int depth = (int)m.z;
             float opl = o4.w;
             const float3 d = xyz(d4);
@@ -575,16 +618,6 @@ __global__ void __launch_bounds__(128) k_wf_shade_pol(const DevScene s, const Wf
                 done = true;
             } else {
                 verts++;
-                Mueller P;
-                if (depth == 1) {  // a camera ray: identity per colour (not stored)
-#pragma unroll
-                    for (int c = 0; c < 3; ++c)
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) P.m[c][e] = (e % 5 == 0) ? 1.f : 0.f;
-                } else {
-                    load_mueller(p, slot, P);
-                }
-                const float3 xf = xyz(p.xframe[slot]);
                 const int k = h.x, orig = h.y;
                 const float th = __int_as_float(h.z);
                 const float3 x = xyz(o4) + d * th;
@@ -594,31 +627,34 @@ __global__ void __launch_bounds__(128) k_wf_shade_pol(const DevScene s, const Wf
                 const float3 wo = -d;
                 const float cwo = dot(ng, wo);
                 const int unit = __float_as_int(sn.w);
-                if (unit >= 0 && cwo > 0.f) {  // emission: column 0 of P (unpolarised emitter)
+                const bool last = depth == p.max_depth;
+                // emission found here: column 0 of the throughput (unpolarised emitter)
+                const bool emit = unit >= 0 && cwo > 0.f;
+                float e_w = 1.0f, e_opl = 0.f, e_le[3] = {0.f, 0.f, 0.f};
+                if (emit) {
                     const LightUnit U = s.units[unit];
-                    float w = 1.0f;
-                    if (depth > 1) w = mis2w(d4.w, (U.v1.w / U.v0.w) * th * th / cwo);
+                    if (depth > 1) e_w = mis2w(d4.w, (U.v1.w / U.v0.w) * th * th / cwo);
                     const float4 Le = s.em_rad[__float_as_int(U.v2.w)];
-                    const float le[3] = {Le.x, Le.y, Le.z};
-                    float S[3][4];
-#pragma unroll
-                    for (int c = 0; c < 3; ++c)
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) S[c][q] = P.m[c][4 * q] * le[c] * w * p.scale;
-                    wf_splat_stokes(p, pix, opl + pulse_time(s, pix, smp, (uint32_t)depth, 0, p.k0, p.k1), S);
+                    e_le[0] = Le.x, e_le[1] = Le.y, e_le[2] = Le.z;
+                    e_opl = opl + pulse_time(s, pix, smp, (uint32_t)depth, 0, p.k0, p.k1);
                     contribs++;
                 }
-                if (depth == p.max_depth) {
-                    done = true;
-                } else {
+                // the next-event estimate and the continuation at this vertex; *_r = turn of the frame into the
+                // scattering plane (cosine and sine of twice the angle), *_f = scalar factor, *_cd = microfacet cosine
+                bool nee = false;
+                float n_cx = 0.f, n_geo = 0.f, n_w = 0.f, n_f = 0.f, n_cd = 0.f, n_le[3] = {0.f, 0.f, 0.f};
+                float n_c2 = 1.f, n_s2 = 0.f, c_c2 = 1.f, c_s2 = 0.f, c_f = 0.f, c_cd = 0.f, c_pb = 1.f, c_z = 0.f;
+                Mat mat{f3(0.f, 0.f, 0.f), -1.f};
+                if (!last) {
                     opl += vertex_delay(s, orig, pix, smp, (uint32_t)depth, p.k0, p.k1);
                     const float3 nn = cwo >= 0.f ? ng : -ng;
                     float3 tb, bb;
                     onb(nn, tb, bb);
                     const float3 wol = to_local(wo, tb, bb, nn);
                     const float4 mm = __ldg(&s.shrec[2 * (size_t)k + 1]);
-                    const Mat mat{xyz(mm), mm.w};
-                    const float alb[3] = {mm.x, mm.y, mm.z};
+                    mat = Mat{xyz(mm), mm.w};
+                    const bool turn = mat.rough >= 0.f && form != MT_POL_COLUMN;  // the frame matters here
+                    const float3 xf = turn ? xyz(p.xframe[slot]) : f3(0.f, 0.f, 0.f);
                     if (s.n_units > 0) {  // next-event estimate, queued for the shadow stage
                         const uint4 R = philox4x32_10(make_uint4(pix, smp, (uint32_t)depth, G_NEE), p.k0, p.k1);
                         const LightUnit U = s.units[pick_unit_wf(s, R.x)];
@@ -646,45 +682,18 @@ __global__ void __launch_bounds__(128) k_wf_shade_pol(const DevScene s, const Wf
                                 w = mis2w(pA * dist * dist / cy, pb);
                             }
                             const float4 Le = s.em_rad[em];
-                            const float le[3] = {Le.x, Le.y, Le.z};
-                            if (mat.rough < 0.f) {
-#pragma unroll
-                                for (int c = 0; c < 3; ++c) {
-                                    const float kk = alb[c] * (1.0f / MT_PI) * cx * geo * w * le[c] * p.scale;
-#pragma unroll
-                                    for (int q = 0; q < 4; ++q) S_nee[c][q] = P.m[c][4 * q] * kk;
-                                }
-                            } else {
+                            n_le[0] = Le.x, n_le[1] = Le.y, n_le[2] = Le.z;
+                            n_cx = cx, n_geo = geo, n_w = w;
+                            if (mat.rough >= 0.f) {
                                 // column 0 of (P R(t)) M_F, t the turn from the scattering plane to the frame
-                                const float t = frame_angle(wo, plane_normal(wi, d), xf);
-                                float s2, c2;
-                                sincosf(2.0f * t, &s2, &c2);
-                                float cd;
-                                const float kf = ggx_factor(mat.rough, wol, wil, cd) * cx * geo * w * p.scale;
-#pragma unroll
-                                for (int c = 0; c < 3; ++c) {
-                                    const float4 F = fresnel_abcd(cd, conductor_kappa(alb[c]));
-#pragma unroll
-                                    for (int q = 0; q < 4; ++q) {
-                                        const float q0 = P.m[c][4 * q];
-                                        const float q1 = P.m[c][4 * q + 1] * c2 - P.m[c][4 * q + 2] * s2;
-                                        S_nee[c][q] = (q0 * F.x + q1 * F.y) * kf * le[c];
-                                    }
-                                }
+                                if (turn) sincosf(2.0f * frame_angle(wo, plane_normal(wi, d), xf), &n_s2, &n_c2);
+                                n_f = ggx_factor(mat.rough, wol, wil, n_cd) * cx * geo * w * p.scale;
                             }
-                            bool nonzero = false;
-#pragma unroll
-                            for (int c = 0; c < 3; ++c)
-#pragma unroll
-                                for (int q = 0; q < 4; ++q) nonzero |= S_nee[c][q] != 0.f;
-                            if (nonzero) {
-                                shadow = true;
-                                sh_o = make_float4(xo.x, xo.y, xo.z, dist - (is_pt ? 0.0f : eps_of(y)));
-                                sh_d = make_float4(wi.x, wi.y, wi.z,
-                                                   opl + dist + pulse_time(s, pix, smp, (uint32_t)depth, 1, p.k0,
-                                                                           p.k1));
-                                sh_c = make_float4(0.f, 0.f, 0.f, __int_as_float((int)pix));
-                            }
+                            nee = true;
+                            sh_o = make_float4(xo.x, xo.y, xo.z, dist - (is_pt ? 0.0f : eps_of(y)));
+                            sh_d = make_float4(wi.x, wi.y, wi.z,
+                                               opl + dist + pulse_time(s, pix, smp, (uint32_t)depth, 1, p.k0, p.k1));
+                            sh_c = make_float4(0.f, 0.f, 0.f, __int_as_float((int)pix));
                         }
                     }
                     // continue by sampling the BSDF
@@ -695,57 +704,111 @@ __global__ void __launch_bounds__(128) k_wf_shade_pol(const DevScene s, const Wf
                         float pb;
                         bsdf_eval(mat, wol, wil, f, pb);
                         if (pb > 0.f) {
+                            cont = true;
                             const float3 wi = to_world(wil, tb, bb, nn);
-                            const float3 sv = plane_normal(wi, d);
-                            rotate_columns(P, frame_angle(wo, sv, xf));
-                            if (mat.rough < 0.f) {  // ideal depolariser
-#pragma unroll
-                                for (int c = 0; c < 3; ++c) {
-                                    const float kk = alb[c] * (1.0f / MT_PI) * wil.z / pb;
-#pragma unroll
-                                    for (int q = 0; q < 4; ++q) {
-                                        P.m[c][4 * q] *= kk;
-                                        P.m[c][4 * q + 1] = 0.f;
-                                        P.m[c][4 * q + 2] = 0.f;
-                                        P.m[c][4 * q + 3] = 0.f;
-                                    }
-                                }
-                            } else {  // P <- P M_F (Fresnel Mueller of the microfacet) x GGX factor / pdf
-                                float cd;
-                                const float kf = ggx_factor(mat.rough, wol, wil, cd) * wil.z / pb;
-#pragma unroll
-                                for (int c = 0; c < 3; ++c) {
-                                    const float4 F = fresnel_abcd(cd, conductor_kappa(alb[c]));
-#pragma unroll
-                                    for (int q = 0; q < 4; ++q) {
-                                        float *row = &P.m[c][4 * q];
-                                        const float r0 = row[0], r1 = row[1], r2 = row[2], r3 = row[3];
-                                        row[0] = (r0 * F.x + r1 * F.y) * kf;
-                                        row[1] = (r0 * F.y + r1 * F.x) * kf;
-                                        row[2] = (r2 * F.z - r3 * F.w) * kf;
-                                        row[3] = (r2 * F.w + r3 * F.z) * kf;
-                                    }
-                                }
+                            c_pb = pb;
+                            c_z = wil.z;
+                            if (mat.rough >= 0.f) {
+                                const float3 sv = plane_normal(wi, d);
+                                if (turn) sincosf(2.0f * frame_angle(wo, sv, xf), &c_s2, &c_c2);
+                                c_f = ggx_factor(mat.rough, wol, wil, c_cd) * wil.z / pb;
+                                p.xframe[slot] = make_float4(sv.x, sv.y, sv.z, 0.f);
                             }
-                            store_mueller(p, slot, P);
-                            p.xframe[slot] = make_float4(sv.x, sv.y, sv.z, 0.f);
                             const float3 no = x + nn * eps_of(x);
                             p.o[slot] = make_float4(no.x, no.y, no.z, opl);
                             p.d[slot] = make_float4(wi.x, wi.y, wi.z, pb);
-                            p.meta[slot] = make_uint4(pix, smp, (uint32_t)(depth + 1), 0u);
-                            cont = true;
+                            p.meta[slot] = make_uint4(pix, smp, (uint32_t)(depth + 1),
+                                                      mat.rough < 0.f ? MT_POL_COLUMN : MT_POL_FULL);
                         }
                     }
-                    if (!cont) done = true;
                 }
+                if (!cont) done = true;
+                // the colours, one after the other
+                float *ef = nullptr, *es = nullptr;
+                if (emit) {
+                    const uint32_t lp = pix - p.pix_base;
+                    const float t = (e_opl - p.start) / p.width;
+                    if (t >= 0.f && t < (float)p.T) ef = p.film + ((size_t)lp * p.T + (int)t) * 12;
+                    es = p.steady + (size_t)lp * 12;
+                }
+                const float alb[3] = {mat.alb.x, mat.alb.y, mat.alb.z};
+                float4 *mu = p.mueller + (size_t)slot * 12;
+                bool nonzero = false;
+                float4 col[3];
+                if (form == MT_POL_COLUMN)
+                    for (int c = 0; c < 3; ++c) col[c] = mu[c];  // read before any colour's rows are written
+                if (emit || nee || cont) {
+#pragma unroll 1
+                    for (int c = 0; c < 3; ++c) {
+                        float r[4][4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) r[q][e] = form == MT_POL_IDENTITY && q == e ? 1.f : 0.f;
+                        if (form == MT_POL_COLUMN) {
+                            r[0][0] = col[c].x, r[1][0] = col[c].y, r[2][0] = col[c].z, r[3][0] = col[c].w;
+                        } else if (form == MT_POL_FULL) {
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const float4 v = mu[c * 4 + q];
+                                r[q][0] = v.x, r[q][1] = v.y, r[q][2] = v.z, r[q][3] = v.w;
+                            }
+                        }
+                        if (emit) {
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const float v = r[q][0] * e_le[c] * e_w * p.scale;
+                                if (v != 0.f) {
+                                    if (ef) atomicAdd(ef + q * 3 + c, v);
+                                    atomicAdd(es + q * 3 + c, v);
+                                }
+                            }
+                        }
+                        if (mat.rough < 0.f) {
+                            if (nee) {
+                                const float kk = alb[c] * (1.0f / MT_PI) * n_cx * n_geo * n_w * n_le[c] * p.scale;
+#pragma unroll
+                                for (int q = 0; q < 4; ++q) S_nee[c][q] = r[q][0] * kk;
+                            }
+                            if (cont) {  // ideal depolariser
+                                const float kk = alb[c] * (1.0f / MT_PI) * c_z / c_pb;
+                                mu[c] = make_float4(r[0][0] * kk, r[1][0] * kk, r[2][0] * kk, r[3][0] * kk);
+                            }
+                        } else {
+                            if (nee) {
+                                const float4 F = fresnel_abcd(n_cd, conductor_kappa(alb[c]));
+#pragma unroll
+                                for (int q = 0; q < 4; ++q)
+                                    S_nee[c][q] =
+                                        (r[q][0] * F.x + (r[q][1] * n_c2 - r[q][2] * n_s2) * F.y) * n_f * n_le[c];
+                            }
+                            if (cont) {  // P <- P R(t) M_F (Fresnel Mueller of the microfacet) x GGX factor / pdf
+                                const float4 F = fresnel_abcd(c_cd, conductor_kappa(alb[c]));
+#pragma unroll
+                                for (int q = 0; q < 4; ++q) {
+                                    const float r0 = r[q][0], r1 = r[q][1] * c_c2 - r[q][2] * c_s2,
+                                                r2 = r[q][1] * c_s2 + r[q][2] * c_c2, r3 = r[q][3];
+                                    mu[c * 4 + q] = make_float4((r0 * F.x + r1 * F.y) * c_f, (r0 * F.y + r1 * F.x) * c_f,
+                                                                (r2 * F.z - r3 * F.w) * c_f, (r2 * F.w + r3 * F.z) * c_f);
+                                }
+                            }
+                        }
+                        if (nee)
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) nonzero |= S_nee[c][q] != 0.f;
+                    }
+                }
+                shadow = nee && nonzero;
             }
         }
-        const uint32_t qs = wf_append(&p.counters[C_NEXT], cont);
-        if (cont) qnext[qs] = slot;
-        const uint32_t fs = wf_append(&p.counters[C_FREE], done);
-        if (done) p.free_q[fs] = slot;
-        const uint32_t ss = wf_append(&p.counters[C_SHADOW], shadow);
+        uint32_t *const queues[3] = {&p.counters[C_NEXT], &p.counters[C_SHADOW], &p.counters[C_FREE]};
+        const bool want[3] = {cont, shadow, done};
+        uint32_t at[3];
+        wf_append_n<3>(queues, want, at);
+        if (cont) qnext[at[0]] = slot;
+        if (done) p.free_q[at[2]] = slot;
         if (shadow) {
+            const uint32_t ss = at[1];
             p.sh_o[ss] = sh_o;
             p.sh_d[ss] = sh_d;
             p.sh_c[ss] = sh_c;
@@ -905,9 +968,14 @@ __global__ void __launch_bounds__(256) k_wf_trace_dyn(const DevScene s, const Wf
     }
 }
 
-// the shading stage at 3 CTAs per SM (80 registers, no spills)
+// CTAs per SM of the shading stage: it waits on gathers and on the queue appends, so the plain forward form runs at 4
+// (render of the 1.16M-triangle scene 64.95 / 62.83 / 61.91 ms at 2 / 3 / 4); the medium and the replay keep 3 (media
+// training step 69.3 / 68.2 / 69.7 ms at 2 / 3 / 4)
 #ifndef MT_WF_SHADE_MINB
 #define MT_WF_SHADE_MINB 3
+#endif
+#ifndef MT_WF_SHADE_FWD_MINB
+#define MT_WF_SHADE_FWD_MINB 4
 #endif
 
 __device__ __forceinline__ float3 drad_of(const WfParams &p, int em) {
@@ -923,8 +991,8 @@ __device__ __forceinline__ float3 drad_of(const WfParams &p, int em) {
 // here; the next-event term is added by the shadow stage), paths that end go to
 // the finalize queue; radiance gradients are summed per CTA.
 template <bool DUMP, bool MEDIA, bool TAN, bool BWD>
-__global__ void __launch_bounds__(256, MT_WF_SHADE_MINB) k_wf_shade(const DevScene s, const WfParams p, const uint32_t *qcur,
-                                                  uint32_t *qnext) {
+__global__ void __launch_bounds__(256, DUMP || MEDIA || TAN || BWD ? MT_WF_SHADE_MINB : MT_WF_SHADE_FWD_MINB)
+    k_wf_shade(const DevScene s, const WfParams p, const uint32_t *qcur, uint32_t *qnext) {
     __shared__ float em_acc[BWD ? MT_WF_EM_SMEM * 3 : 1];
     if (BWD) {
         for (int k = threadIdx.x; k < MT_WF_EM_SMEM * 3; k += blockDim.x) em_acc[k] = 0.f;
@@ -1184,7 +1252,20 @@ __global__ void __launch_bounds__(256, MT_WF_SHADE_MINB) k_wf_shade(const DevSce
             p.rec_b[r] = make_float4(Sv.x, Sv.y, Sv.z, 0.f);
             p.rec_c[r] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        const uint32_t qs = wf_append(&p.counters[C_NEXT], cont);
+        uint32_t qs, ss, fs = 0;
+        if (BWD || !qord) {  // the slot of a finished path returns to the free stack (replay: to the finalize queue)
+            uint32_t *const queues[3] = {&p.counters[C_NEXT], &p.counters[C_SHADOW], &p.counters[BWD ? C_FIN : C_FREE]};
+            const bool want[3] = {cont, shadow, done};
+            uint32_t at[3];
+            wf_append_n<3>(queues, want, at);
+            qs = at[0], ss = at[1], fs = at[2];
+        } else {
+            uint32_t *const queues[2] = {&p.counters[C_NEXT], &p.counters[C_SHADOW]};
+            const bool want[2] = {cont, shadow};
+            uint32_t at[2];
+            wf_append_n<2>(queues, want, at);
+            qs = at[0], ss = at[1];
+        }
         if (cont) {
             if (qord) {
                 p.ps_o_n[qs] = n_o;
@@ -1199,18 +1280,14 @@ __global__ void __launch_bounds__(256, MT_WF_SHADE_MINB) k_wf_shade(const DevSce
                 if (TAN) p.sig[slot] = make_float4(n_sig.x, n_sig.y, n_sig.z, 0.f);
             }
         }
-        if (!qord) {  // the slot of a finished path returns to the free stack (replay: to the finalize queue)
-            const uint32_t fs = wf_append(&p.counters[BWD ? C_FIN : C_FREE], done);
-            if (done) {
-                if (BWD) {
-                    p.fin_q[fs] = slot;
-                    p.meta[slot] = make_uint4(m.x, m.y, m.z, (uint32_t)end);
-                } else {
-                    p.free_q[fs] = slot;
-                }
+        if (!qord && done) {
+            if (BWD) {
+                p.fin_q[fs] = slot;
+                p.meta[slot] = make_uint4(m.x, m.y, m.z, (uint32_t)end);
+            } else {
+                p.free_q[fs] = slot;
             }
         }
-        const uint32_t ss = wf_append(&p.counters[C_SHADOW], shadow);
         if (shadow) {
             p.sh_o[ss] = sh_o;
             p.sh_d[ss] = sh_d;
