@@ -228,6 +228,29 @@ __global__ void k_check_delays(const float *tau, int n, int *bad) {
         if (!(tau[i] >= 0.0f) || !isfinite(tau[i])) atomicOr(bad, 1);
 }
 
+// pairs of triangle records for trace_flat: the missing partner of an odd last triangle is a point (never hit)
+__global__ void k_flat_pairs(const float4 *tris, int n, float4 *flat) {
+    for (int i = threadIdx.x; i < 3 * ((n + 1) / 2); i += blockDim.x) {
+        const int pair = i / 3, a = i - 3 * pair;
+        const float4 x = tris[3 * (2 * pair) + a];
+        const float4 y = 2 * pair + 1 < n ? tris[3 * (2 * pair + 1) + a] : make_float4(0.f, 0.f, 0.f, __int_as_float(0x7fffffff));
+        flat[2 * i] = make_float4(x.x, y.x, x.y, y.y);
+        flat[2 * i + 1] = make_float4(x.z, y.z, x.w, y.w);
+    }
+}
+
+// the plane words of each triangle's leaf, from the nodes that refer to the leaves
+__global__ void k_flat_boxes(const uint4 *nodes, int n_nodes, int n, uint4 *box) {
+    for (int i = threadIdx.x; i < 2 * n_nodes; i += blockDim.x) {
+        const uint4 a = nodes[2 * (i >> 1)], b = nodes[2 * (i >> 1) + 1];
+        const uint32_t ref = i & 1 ? b.w : b.z;
+        if (!(ref & 0x80000000u) || ref == MT_EMPTY_REF) continue;
+        const uint4 w = i & 1 ? make_uint4(a.w, b.x, b.y, 0u) : make_uint4(a.x, a.y, a.z, 0u);
+        const int first = (int)(ref & 0x1FFFFFFFu), last = first + (int)((ref >> 29) & 3u);
+        for (int k = first; k <= last && k < n; ++k) box[k] = w;
+    }
+}
+
 __global__ void k_leaf_of(const float4 *tris, int n, int32_t *leaf_of) {
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
         leaf_of[__float_as_int(tris[3 * k].w)] = k;
@@ -555,6 +578,23 @@ static mt_status scene_create_impl(const float *tris, int64_t n, const mt_materi
     float4 *shrec;
     MT_TRY(al.alloc(&shrec, (size_t)2 * n, "shading records"));
     k_shading_records<<<g, 256, 0, st>>>(sc->bvh.tris, mats4, tri_unit, (int)n, shrec);
+    // Small scenes traced triangle by triangle (trace_flat): in a medium, and where the tree's expected walk (its SAH
+    // cost) is long for so few triangles.  Frames of 128x128 px, 32 spp, depth 6, tree / loop in the persistent form:
+    // in a medium, closed rooms and boxes of 13 to 37 triangles 1022 / 890 to 2325 / 1457 us, random open meshes of 6,
+    // 16, 36, 48, 64 triangles 917 / 741, 1174 / 881, 1436 / 1290, 1476 / 1484, 1560 / 1710, but planes of 2 to 6
+    // triangles 697 / 977 to 1623 / 1828; without one, 20-triangle sphere (SAH cost 13.6) 891 / 471, 37-triangle room
+    // (14.1) 601 / 598, Cornell box (14.5) 611 / 596, 25-triangle room (10.2) 439 / 493, 36 random triangles (5.0) 188 /
+    // 242.  Small frames gain more: Cornell box 64x64, 16 spp 135 / 100.
+    if (n >= 8 && n <= 48 && (med || sc->bvh.sah >= 13.0)) {
+        float4 *flat;
+        MT_TRY(al.alloc(&flat, (size_t)6 * ((n + 1) / 2), "triangle pairs"));
+        uint4 *box;
+        MT_TRY(al.alloc(&box, (size_t)n, "triangle leaf boxes"));
+        k_flat_pairs<<<1, 128, 0, st>>>(sc->bvh.tris, (int)n, flat);
+        k_flat_boxes<<<1, 128, 0, st>>>(sc->bvh.nodes, sc->bvh.n_nodes, (int)n, box);
+        D.flat = flat;
+        D.flat_box = box;
+    }
     D.mats = mats4;
     D.tri_unit = tri_unit;
     D.leaf_of = leaf_of;

@@ -265,6 +265,8 @@ struct DevScene {
     const uint4 *nodes;    // 2 x uint4 per internal node
     const uint4 *wnodes;   // 5 x uint4 per 8-wide node (root = node 0)
     const float4 *tris;    // 3 x float4 per leaf-ordered triangle: row a = (v0[a], v1[a], v2[a], original index)
+    const float4 *flat;    // triangle pairs of a small scene (see trace_flat), else null
+    const uint4 *flat_box; // and its leaves' boxes per triangle
     const float4 *mats;    // per original triangle: albedo, w = GGX roughness or -1 (Lambert)
     const int32_t *tri_unit; // per original triangle: light unit or -1
     const int32_t *leaf_of;  // per original triangle: its leaf-order index
@@ -337,12 +339,12 @@ __device__ __forceinline__ float density_at(const DevScene &s, float3 p) {
         v[0] = D(x0, y0, z0), v[1] = D(x1, y0, z0), v[2] = D(x0, y1, z0), v[3] = D(x1, y1, z0);
         v[4] = D(x0, y0, z1), v[5] = D(x1, y0, z1), v[6] = D(x0, y1, z1), v[7] = D(x1, y1, z1);
     }
-    const float c00 = v[0] * (1.f - fx) + v[1] * fx;
-    const float c10 = v[2] * (1.f - fx) + v[3] * fx;
-    const float c01 = v[4] * (1.f - fx) + v[5] * fx;
-    const float c11 = v[6] * (1.f - fx) + v[7] * fx;
-    const float c0 = c00 * (1.f - fy) + c10 * fy, c1 = c01 * (1.f - fy) + c11 * fy;
-    return c0 * (1.f - fz) + c1 * fz;
+    // contraction spelled out, so that every kernel rounds the same way
+    auto mix = [](float a, float b, float f) { return fmaf(a, 1.f - f, b * f); };
+    const float c00 = mix(v[0], v[1], fx), c10 = mix(v[2], v[3], fx);
+    const float c01 = mix(v[4], v[5], fx), c11 = mix(v[6], v[7], fx);
+    const float c0 = mix(c00, c10, fy), c1 = mix(c01, c11, fy);
+    return mix(c0, c1, fz);
 }
 
 // overlap of the ray with the medium box, clipped to [0, tmax]

@@ -80,7 +80,7 @@ __device__ __forceinline__ int pick_unit(const DevScene &s, uint32_t u) {
     return lo;
 }
 
-template <int MODE, bool MEDIA, bool CNT, bool AGG>
+template <int MODE, bool MEDIA, bool CNT, bool AGG, bool FLAT>
 struct Tracer {
     const DevScene &s;
     const RenderParams &p;
@@ -273,7 +273,7 @@ struct Tracer {
         const float tmax = dist - (is_pt ? 0.0f : eps_of(y));
         cnt.rays++;
         const RayT sr = make_ray(s, xo, wi);
-        if (trace_any<CNT>(s, sr, tmax, cnt.tc)) return;
+        if (scene_any<CNT, FLAT>(s, sr, tmax, cnt.tc)) return;
         float Tr = 1.0f;
         if (MEDIA) {
             bool ok;
@@ -326,7 +326,7 @@ struct Tracer {
         float th;
         int orig;
         cnt.rays++;
-        const int k = trace_closest<CNT>(s, r, INFINITY, th, orig, cnt.tc);
+        const int k = scene_closest<CNT, FLAT>(s, r, INFINITY, th, orig, cnt.tc);
         if (MEDIA) {
             float ma, mb;
             const float tsurf = k >= 0 ? th : 1e30f;
@@ -431,7 +431,7 @@ struct Tracer {
     }
 };
 
-template <int MODE, bool MEDIA, bool CNT, bool AGG>
+template <int MODE, bool MEDIA, bool CNT, bool AGG, bool FLAT>
 __global__ void __launch_bounds__(256, MT_MINB_OF(MODE, MEDIA)) k_render(const DevScene s, const RenderParams p) {
     extern __shared__ float4 smem4[];
     float *smem = reinterpret_cast<float *>(smem4);
@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(256, MT_MINB_OF(MODE, MEDIA)) k_render(const D
         if (threadIdx.x == 0) s_med = 0.f;
         __syncthreads();
     }
-    Tracer<MODE, MEDIA, CNT, AGG> tr{s, p, hist, steady_s, em_acc, s_med, cnt, vrec, Rng{p.k0, p.k1}};
+    Tracer<MODE, MEDIA, CNT, AGG, FLAT> tr{s, p, hist, steady_s, em_acc, s_med, cnt, vrec, Rng{p.k0, p.k1}};
     for (;;) {
         // the warp claims its next tile
         int tile = 0;
@@ -553,9 +553,9 @@ __global__ void __launch_bounds__(256, MT_MINB_OF(MODE, MEDIA)) k_render(const D
     }
 }
 
-template <int MODE, bool MEDIA, bool CNT, bool AGG>
-mt_status launch_one(const DevScene &s, const RenderParams &p, const LaunchCfg &cfg, cudaStream_t st) {
-    auto kern = k_render<MODE, MEDIA, CNT, AGG>;
+template <int MODE, bool MEDIA, bool CNT, bool AGG, bool FLAT>
+mt_status launch_form(const DevScene &s, const RenderParams &p, const LaunchCfg &cfg, cudaStream_t st) {
+    auto kern = k_render<MODE, MEDIA, CNT, AGG, FLAT>;
     const size_t smem = cfg.smem_bytes;
     MT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
@@ -570,6 +570,21 @@ mt_status launch_one(const DevScene &s, const RenderParams &p, const LaunchCfg &
     kern<<<grid, cfg.threads, smem, st>>>(s, p);
     MT_CUDA_TRY(cudaGetLastError());
     return MT_OK;
+}
+
+// Small scenes test every triangle in turn when a warp's tile holds enough paths for its lanes to share the work; with
+// fewer lanes the tree's shorter walk is as fast (Cornell box, 64x64 px, 16 spp: 109 -> 79 us; 23x37 px, 1 spp, one
+// path per warp: 37 us in the tree, 39 triangle by triangle).
+#ifndef MT_FLAT_LANES
+#define MT_FLAT_LANES 8
+#endif
+template <int MODE, bool MEDIA, bool CNT, bool AGG>
+mt_status launch_one(const DevScene &s, const RenderParams &p, const LaunchCfg &cfg, cudaStream_t st) {
+    if constexpr (!CNT && !AGG && MODE != MODE_DUMP) {
+        if (s.flat && (long long)p.tile_px * p.spp >= MT_FLAT_LANES)
+            return launch_form<MODE, MEDIA, CNT, AGG, true>(s, p, cfg, st);
+    }
+    return launch_form<MODE, MEDIA, CNT, AGG, false>(s, p, cfg, st);
 }
 
 template <int MODE, bool MEDIA, bool CNT>

@@ -199,7 +199,8 @@ __device__ __forceinline__ bool tri_hit(const RayT &r, const float4 *T, float &t
     if (min3f(U, V, W) < 0.f && max3f(U, V, W) > 0.f) return false;
     const float det = U + V + W;
     if (det == 0.f) return false;
-    const float Tn = U * (r.Sz * Akz) + V * (r.Sz * Bkz) + W * (r.Sz * Ckz);
+    // contraction spelled out, so that every kernel and trace_flat round the same way
+    const float Tn = fmaf(W, r.Sz * Ckz, fmaf(U, r.Sz * Akz, V * (r.Sz * Bkz)));
     if (det > 0.f ? Tn <= 0.f : Tn >= 0.f) return false;
     t = Tn / det;
     return true;
@@ -329,6 +330,154 @@ __device__ __forceinline__ bool trace_any(const DevScene &s, const RayT &r, floa
         --sp;
         ref = st_ref[sp];
     }
+}
+
+// ---------------------------------------------------------------------------
+// Scenes of a few triangles (the rule is where s.flat is built): every triangle in
+// turn instead of the tree, two per step in packed arithmetic.  All lanes of a warp do the same
+// work, where in the tree of the 36-triangle box a lane in nine instructions of
+// ten waits for another's node or leaf; the steps are independent, so few warps
+// hide their latency.  The hit is the smallest (t, original index) all the same,
+// from the same operations in the same order as tri_hit.  A ray almost in the
+// plane of a triangle can pass the edge tests by rounding far from it; the tree
+// never tests such a triangle, because the ray misses its leaf's box.  So the
+// hit found is checked against the box of its leaf, and a ray that fails goes
+// through the tree (a hit that passes is the tree's own: its ancestors' boxes
+// contain the leaf's, and no triangle is nearer).
+// Records (s.flat, leaf order, built at scene creation): per pair of triangles
+// and axis a 32-byte row (v0, v0', v1, v1', v2, v2', index, index'); s.flat_box:
+// per triangle the three plane words of its leaf.
+// ---------------------------------------------------------------------------
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pk(float a, float b) {
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ void upk(f32x2 v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+struct FlatRow {
+    f32x2 v0, v1, v2;
+    int id0, id1;
+};
+__device__ __forceinline__ FlatRow ld_flat(const float4 *p) {
+    FlatRow r;
+    float a, b, c, d, e, f, g, h;
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(a), "=f"(b), "=f"(c), "=f"(d), "=f"(e), "=f"(f), "=f"(g), "=f"(h)
+        : "l"(p));
+    r.v0 = pk(a, b);
+    r.v1 = pk(c, d);
+    r.v2 = pk(e, f);
+    r.id0 = __float_as_int(g);
+    r.id1 = __float_as_int(h);
+    return r;
+}
+
+// the tests of tri_hit after the edge functions
+__device__ __forceinline__ bool flat_hit(float U, float V, float W, float det, float Tn, float &t) {
+    if (min3f(U, V, W) < 0.f && max3f(U, V, W) > 0.f) return false;
+    if (det == 0.f) return false;
+    if (det > 0.f ? Tn <= 0.f : Tn >= 0.f) return false;
+    t = Tn / det;
+    return true;
+}
+
+// leaf-order index of the closest hit or, ANY, of any hit; -1: none
+template <bool ANY>
+__device__ __forceinline__ int trace_flat(const DevScene &s, const RayT &r, float tmax, float &t_out, int &orig_out) {
+    const float4 *px = s.flat + 2 * r.kx, *py = s.flat + 2 * r.ky, *pz = s.flat + 2 * r.kz;
+    const f32x2 ox = pk(r.ok.x, r.ok.x), oy = pk(r.ok.y, r.ok.y), oz = pk(r.ok.z, r.ok.z);
+    const f32x2 m1 = pk(-1.0f, -1.0f), nSx = pk(-r.Sx, -r.Sx), nSy = pk(-r.Sy, -r.Sy), Sz = pk(r.Sz, r.Sz);
+    float tbest = tmax;
+    int best_k = -1, best_id = 0x7fffffff;
+    const int n = s.n_tris;
+    for (int k = 0; k < n; k += 2, px += 6, py += 6, pz += 6) {
+        const FlatRow X = ld_flat(px), Y = ld_flat(py), Z = ld_flat(pz);
+        const f32x2 Akz = sub2(Z.v0, oz), Bkz = sub2(Z.v1, oz), Ckz = sub2(Z.v2, oz);
+        const f32x2 Ax = fma2(nSx, Akz, sub2(X.v0, ox)), Ay = fma2(nSy, Akz, sub2(Y.v0, oy));
+        const f32x2 Bx = fma2(nSx, Bkz, sub2(X.v1, ox)), By = fma2(nSy, Bkz, sub2(Y.v1, oy));
+        const f32x2 Cx = fma2(nSx, Ckz, sub2(X.v2, ox)), Cy = fma2(nSy, Ckz, sub2(Y.v2, oy));
+        // products and difference each rounded, as in tri_hit: a packed subtraction of packed products would be
+        // contracted, an FMA with -1 is not
+        const f32x2 U = fma2(mul2(Cy, Bx), m1, mul2(Cx, By));
+        const f32x2 V = fma2(mul2(Ay, Cx), m1, mul2(Ax, Cy));
+        const f32x2 W = fma2(mul2(By, Ax), m1, mul2(Bx, Ay));
+        const f32x2 det = add2(add2(U, V), W);
+        const f32x2 T = fma2(W, mul2(Sz, Ckz), fma2(U, mul2(Sz, Akz), mul2(V, mul2(Sz, Bkz))));
+        float u[2], v[2], w[2], d[2], tn[2];
+        upk(U, u[0], u[1]);
+        upk(V, v[0], v[1]);
+        upk(W, w[0], w[1]);
+        upk(det, d[0], d[1]);
+        upk(T, tn[0], tn[1]);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            float t;
+            if (flat_hit(u[j], v[j], w[j], d[j], tn[j], t) && t < tmax) {
+                if (ANY) return k + j;
+                const int id = j ? Z.id1 : Z.id0;
+                if (t < tbest || (t == tbest && id < best_id)) {
+                    tbest = t;
+                    best_k = k + j;
+                    best_id = id;
+                }
+            }
+        }
+    }
+    t_out = tbest;
+    orig_out = best_id;
+    return best_k;
+}
+
+// whether the ray enters the box of triangle k's leaf up to tmax, as the tree tests it
+__device__ __forceinline__ bool flat_in_box(const DevScene &s, const RayT &r, int k, float tmax) {
+    const uint4 w = __ldg(&s.flat_box[k]);
+    float tn, tf;
+    slab(r, w.x, w.y, w.z, tmax, tn, tf);
+    return tn <= tf;
+}
+
+// the scene's own way: all triangles (FLAT, scenes that have s.flat) or the binary tree
+template <bool CNT, bool FLAT>
+__device__ __forceinline__ int scene_closest(const DevScene &s, const RayT &r, float tmax, float &t_out, int &orig_out,
+                                             TraceCnt &cnt) {
+    if (FLAT) {
+        const int k = trace_flat<false>(s, r, tmax, t_out, orig_out);
+        if (k < 0 || flat_in_box(s, r, k, t_out)) return k;
+    }
+    return trace_closest<CNT>(s, r, tmax, t_out, orig_out, cnt);
+}
+template <bool CNT, bool FLAT>
+__device__ __forceinline__ bool scene_any(const DevScene &s, const RayT &r, float tmax, TraceCnt &cnt) {
+    if (FLAT) {
+        float t;
+        int id;
+        const int k = trace_flat<true>(s, r, tmax, t, id);
+        if (k < 0) return false;
+        if (flat_in_box(s, r, k, tmax)) return true;
+    }
+    return trace_any<CNT>(s, r, tmax, cnt);
 }
 
 // ---------------------------------------------------------------------------

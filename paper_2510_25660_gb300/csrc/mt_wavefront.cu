@@ -401,10 +401,16 @@ __global__ void __launch_bounds__(256) k_wf_generate(const DevScene s, const WfP
 #ifndef MT_WF_MEDIA_MINB
 #define MT_WF_MEDIA_MINB 5
 #endif
+// small scenes triangle by triangle: media training step in the 36-triangle box 69.0 ms in the tree, 65.5 / 60.4 / 63.3
+// at 3 / 4 / 5 CTAs per SM
+#ifndef MT_WF_FLAT_MINB
+#define MT_WF_FLAT_MINB 4
+#endif
+#define MT_WF_MINB(MEDIA, FLAT) ((FLAT) ? MT_WF_FLAT_MINB : (MEDIA) ? MT_WF_MEDIA_MINB : MT_WF_TRACE_MINB)
 
 // hit record: (leaf-order triangle or -1, original triangle, t bits, 1 if the
 // path scatters in the medium at t before reaching that surface)
-template <bool WIDE, bool CNT, bool MEDIA>
+template <bool WIDE, bool CNT, bool MEDIA, bool FLAT>
 __device__ __forceinline__ void ext_rays(const DevScene &s, const WfParams &p, const uint32_t *qcur, TraceCnt &tc,
                                          uint32_t &rays) {
     const uint32_t n = p.counters[C_CUR];
@@ -433,7 +439,7 @@ __device__ __forceinline__ void ext_rays(const DevScene &s, const WfParams &p, c
         if (WIDE) {
             k = live ? trace_wide<false, CNT>(s, r, INFINITY, t, orig, tc) : -1;
         } else {
-            k = live ? trace_closest<CNT>(s, r, INFINITY, t, orig, tc) : -1;
+            k = live ? scene_closest<CNT, FLAT>(s, r, INFINITY, t, orig, tc) : -1;
         }
         if (live) {
             int collided = 0;
@@ -472,12 +478,12 @@ __device__ __forceinline__ void ext_rays(const DevScene &s, const WfParams &p, c
     }
 }
 
-template <bool WIDE, bool CNT, bool MEDIA>
-__global__ void __launch_bounds__(256, MEDIA ? MT_WF_MEDIA_MINB : MT_WF_TRACE_MINB)
+template <bool WIDE, bool CNT, bool MEDIA, bool FLAT>
+__global__ void __launch_bounds__(256, MT_WF_MINB(MEDIA, FLAT))
     k_wf_extend(const DevScene s, const WfParams p, const uint32_t *qcur) {
     TraceCnt tc{0, 0};
     uint32_t rays = 0;
-    ext_rays<WIDE, CNT, MEDIA>(s, p, qcur, tc, rays);
+    ext_rays<WIDE, CNT, MEDIA, FLAT>(s, p, qcur, tc, rays);
     warp_count(&s.counters[3], rays);
     if (CNT) {
         warp_count(&s.counters[4], tc.nodes);
@@ -1311,7 +1317,7 @@ __global__ void __launch_bounds__(256, DUMP || MEDIA || TAN || BWD ? MT_WF_SHADE
     if (BWD) em_grad_flush(p, em_acc, s.n_em);
 }
 
-template <bool DUMP, bool CNT, bool WIDE, bool MEDIA, bool BWD>
+template <bool DUMP, bool CNT, bool WIDE, bool MEDIA, bool BWD, bool FLAT>
 __device__ __forceinline__ void sh_rays(const DevScene &s, const WfParams &p, uint32_t n, float *em_acc,
                                         TraceCnt &tc, uint32_t &rays, uint32_t &contribs) {
     const int lane = threadIdx.x & 31;
@@ -1329,7 +1335,7 @@ __device__ __forceinline__ void sh_rays(const DevScene &s, const WfParams &p, ui
             float t_unused;
             int id_unused;
             const bool occluded = WIDE ? trace_wide<true, CNT>(s, r, o.w, t_unused, id_unused, tc) >= 0
-                                       : trace_any<CNT>(s, r, o.w, tc);
+                                       : scene_any<CNT, FLAT>(s, r, o.w, tc);
             if (!occluded) {
                 const float4 c = p.sh_c[i];
                 const uint32_t pix = (uint32_t)__float_as_int(c.w);
@@ -1372,8 +1378,8 @@ __device__ __forceinline__ void sh_rays(const DevScene &s, const WfParams &p, ui
 }
 
 // shadow rays of this iteration's shading; n_idx names the counter that holds their number
-template <bool DUMP, bool CNT, bool WIDE, bool MEDIA, bool BWD>
-__global__ void __launch_bounds__(256, MEDIA ? MT_WF_MEDIA_MINB : MT_WF_TRACE_MINB)
+template <bool DUMP, bool CNT, bool WIDE, bool MEDIA, bool BWD, bool FLAT>
+__global__ void __launch_bounds__(256, MT_WF_MINB(MEDIA, FLAT))
     k_wf_shadow(const DevScene s, const WfParams p, int n_idx) {
     __shared__ float em_acc[BWD ? MT_WF_EM_SMEM * 3 : 1];
     if (BWD) {
@@ -1382,7 +1388,7 @@ __global__ void __launch_bounds__(256, MEDIA ? MT_WF_MEDIA_MINB : MT_WF_TRACE_MI
     }
     TraceCnt tc{0, 0};
     uint32_t rays = 0, contribs = 0;
-    sh_rays<DUMP, CNT, WIDE, MEDIA, BWD>(s, p, p.counters[n_idx], em_acc, tc, rays, contribs);
+    sh_rays<DUMP, CNT, WIDE, MEDIA, BWD, FLAT>(s, p, p.counters[n_idx], em_acc, tc, rays, contribs);
     warp_count(&s.counters[3], rays);
     warp_count(&s.counters[2], contribs);
     if (CNT) {
@@ -1396,13 +1402,13 @@ __global__ void __launch_bounds__(256, MEDIA ? MT_WF_MEDIA_MINB : MT_WF_TRACE_MI
 // rays that the previous iteration's shading queued (they are independent of
 // each other), so that warps that find the extension queue drained trace
 // shadow rays instead of idling in the tail of the pass.
-template <bool WIDE, bool CNT, bool MEDIA, bool DUMP>
-__global__ void __launch_bounds__(256, MEDIA ? MT_WF_MEDIA_MINB : MT_WF_TRACE_MINB)
+template <bool WIDE, bool CNT, bool MEDIA, bool DUMP, bool FLAT>
+__global__ void __launch_bounds__(256, MT_WF_MINB(MEDIA, FLAT))
     k_wf_trace(const DevScene s, const WfParams p, const uint32_t *qcur) {
     TraceCnt tc{0, 0};
     uint32_t rays = 0, contribs = 0;
-    ext_rays<WIDE, CNT, MEDIA>(s, p, qcur, tc, rays);
-    sh_rays<DUMP, CNT, WIDE, MEDIA, false>(s, p, p.counters[C_SH_N], nullptr, tc, rays, contribs);
+    ext_rays<WIDE, CNT, MEDIA, FLAT>(s, p, qcur, tc, rays);
+    sh_rays<DUMP, CNT, WIDE, MEDIA, false, FLAT>(s, p, p.counters[C_SH_N], nullptr, tc, rays, contribs);
     warp_count(&s.counters[3], rays);
     warp_count(&s.counters[2], contribs);
     if (CNT) {
@@ -1564,6 +1570,9 @@ mt_status mt_launch_wavefront(const DevScene &s, const WfParams &p0, int num_sms
         out->used = true;
     }
     const int grid = num_sms * 8;
+    // small scenes in a medium: every triangle in turn (not in the counting, wide and dump forms); without a medium the
+    // full queues hide the tree's divergence better (Cornell box, 128x128 px, 32 spp: 783 us against 811)
+    const bool flat = s.flat != nullptr && s.has_medium;
     k_wf_init<<<std::max(1, std::min(grid, (int)((p.P + 255) / 256))), 256, 0, st>>>(p.qmode ? nullptr : p.free_q, p.P, p.counters,
                                                                                     p.next_path);
     MT_CUDA_TRY(cudaGetLastError());
@@ -1575,14 +1584,15 @@ mt_status mt_launch_wavefront(const DevScene &s, const WfParams &p0, int num_sms
         const bool wide = p.wide && !media && !p.bwd;
         if (!MT_WF_FUSE || p.bwd || p.mueller || dyn || dump) return MT_OK;
         if (media) {
-            if (counters) k_wf_shadow<false, true, false, true, false><<<grid, 256, 0, st>>>(s, p, C_SH_N);
-            else k_wf_shadow<false, false, false, true, false><<<grid, 256, 0, st>>>(s, p, C_SH_N);
+            if (counters) k_wf_shadow<false, true, false, true, false, false><<<grid, 256, 0, st>>>(s, p, C_SH_N);
+            else if (flat) k_wf_shadow<false, false, false, true, false, true><<<grid, 256, 0, st>>>(s, p, C_SH_N);
+            else k_wf_shadow<false, false, false, true, false, false><<<grid, 256, 0, st>>>(s, p, C_SH_N);
         } else if (wide) {
-            if (counters) k_wf_shadow<false, true, true, false, false><<<grid, 256, 0, st>>>(s, p, C_SH_N);
-            else k_wf_shadow<false, false, true, false, false><<<grid, 256, 0, st>>>(s, p, C_SH_N);
+            if (counters) k_wf_shadow<false, true, true, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SH_N);
+            else k_wf_shadow<false, false, true, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SH_N);
         } else {
-            if (counters) k_wf_shadow<false, true, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SH_N);
-            else k_wf_shadow<false, false, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SH_N);
+            if (counters) k_wf_shadow<false, true, false, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SH_N);
+            else k_wf_shadow<false, false, false, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SH_N);
         }
         MT_CUDA_TRY(cudaGetLastError());
         *launches += 2;
@@ -1616,24 +1626,26 @@ mt_status mt_launch_wavefront(const DevScene &s, const WfParams &p0, int num_sms
             else k_wf_trace_dyn<false, false><<<grid, 256, 0, st>>>(s, p, qa);
         } else if (fused) {
             if (media) {
-                if (counters) k_wf_trace<false, true, true, false><<<grid, 256, 0, st>>>(s, p, qext);
-                else k_wf_trace<false, false, true, false><<<grid, 256, 0, st>>>(s, p, qext);
+                if (counters) k_wf_trace<false, true, true, false, false><<<grid, 256, 0, st>>>(s, p, qext);
+                else if (flat) k_wf_trace<false, false, true, false, true><<<grid, 256, 0, st>>>(s, p, qext);
+                else k_wf_trace<false, false, true, false, false><<<grid, 256, 0, st>>>(s, p, qext);
             } else if (wide) {
-                if (counters) k_wf_trace<true, true, false, false><<<grid, 256, 0, st>>>(s, p, qext);
-                else k_wf_trace<true, false, false, false><<<grid, 256, 0, st>>>(s, p, qext);
+                if (counters) k_wf_trace<true, true, false, false, false><<<grid, 256, 0, st>>>(s, p, qext);
+                else k_wf_trace<true, false, false, false, false><<<grid, 256, 0, st>>>(s, p, qext);
             } else {
-                if (counters) k_wf_trace<false, true, false, false><<<grid, 256, 0, st>>>(s, p, qext);
-                else k_wf_trace<false, false, false, false><<<grid, 256, 0, st>>>(s, p, qext);
+                if (counters) k_wf_trace<false, true, false, false, false><<<grid, 256, 0, st>>>(s, p, qext);
+                else k_wf_trace<false, false, false, false, false><<<grid, 256, 0, st>>>(s, p, qext);
             }
         } else if (media) {
-            if (counters) k_wf_extend<false, true, true><<<grid, 256, 0, st>>>(s, p, qext);
-            else k_wf_extend<false, false, true><<<grid, 256, 0, st>>>(s, p, qext);
+            if (counters) k_wf_extend<false, true, true, false><<<grid, 256, 0, st>>>(s, p, qext);
+            else if (flat) k_wf_extend<false, false, true, true><<<grid, 256, 0, st>>>(s, p, qext);
+            else k_wf_extend<false, false, true, false><<<grid, 256, 0, st>>>(s, p, qext);
         } else if (wide) {
-            if (counters) k_wf_extend<true, true, false><<<grid, 256, 0, st>>>(s, p, qext);
-            else k_wf_extend<true, false, false><<<grid, 256, 0, st>>>(s, p, qext);
+            if (counters) k_wf_extend<true, true, false, false><<<grid, 256, 0, st>>>(s, p, qext);
+            else k_wf_extend<true, false, false, false><<<grid, 256, 0, st>>>(s, p, qext);
         } else {
-            if (counters) k_wf_extend<false, true, false><<<grid, 256, 0, st>>>(s, p, qext);
-            else k_wf_extend<false, false, false><<<grid, 256, 0, st>>>(s, p, qext);
+            if (counters) k_wf_extend<false, true, false, false><<<grid, 256, 0, st>>>(s, p, qext);
+            else k_wf_extend<false, false, false, false><<<grid, 256, 0, st>>>(s, p, qext);
         }
         if (streamed) {
             k_wf_bands<<<1, 256, 0, st>>>(p, (uint32_t)iter);
@@ -1669,11 +1681,12 @@ mt_status mt_launch_wavefront(const DevScene &s, const WfParams &p0, int num_sms
             k_wf_shadow_pol<<<grid, 256, 0, st>>>(s, p);
         } else if (p.bwd) {
             if (media) {
-                if (counters) k_wf_shadow<false, true, false, true, true><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
-                else k_wf_shadow<false, false, false, true, true><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+                if (counters) k_wf_shadow<false, true, false, true, true, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+                else if (flat) k_wf_shadow<false, false, false, true, true, true><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+                else k_wf_shadow<false, false, false, true, true, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
             } else {
-                if (counters) k_wf_shadow<false, true, false, false, true><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
-                else k_wf_shadow<false, false, false, false, true><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+                if (counters) k_wf_shadow<false, true, false, false, true, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+                else k_wf_shadow<false, false, false, false, true, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
             }
             k_wf_finalize<<<grid, 256, s.n_tris <= MT_FIN_SMEM_TRIS ? 3 * (size_t)s.n_tris * sizeof(float) : 0, st>>>(s, p);
             *launches += 1;
@@ -1682,26 +1695,26 @@ mt_status mt_launch_wavefront(const DevScene &s, const WfParams &p0, int num_sms
             else k_wf_trace_dyn<true, false><<<grid, 256, 0, st>>>(s, p, qa);
         } else if (media) {
             if (dump) {
-                if (counters) k_wf_shadow<true, true, false, true, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
-                else k_wf_shadow<true, false, false, true, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+                if (counters) k_wf_shadow<true, true, false, true, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+                else k_wf_shadow<true, false, false, true, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
             } else {
-                if (counters) k_wf_shadow<false, true, false, true, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
-                else k_wf_shadow<false, false, false, true, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+                if (counters) k_wf_shadow<false, true, false, true, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+                else k_wf_shadow<false, false, false, true, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
             }
         } else if (wide) {
             if (dump) {
-                if (counters) k_wf_shadow<true, true, true, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
-                else k_wf_shadow<true, false, true, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+                if (counters) k_wf_shadow<true, true, true, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+                else k_wf_shadow<true, false, true, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
             } else {
-                if (counters) k_wf_shadow<false, true, true, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
-                else k_wf_shadow<false, false, true, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+                if (counters) k_wf_shadow<false, true, true, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+                else k_wf_shadow<false, false, true, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
             }
         } else if (dump) {
-            if (counters) k_wf_shadow<true, true, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
-            else k_wf_shadow<true, false, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+            if (counters) k_wf_shadow<true, true, false, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+            else k_wf_shadow<true, false, false, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
         } else {
-            if (counters) k_wf_shadow<false, true, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
-            else k_wf_shadow<false, false, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+            if (counters) k_wf_shadow<false, true, false, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+            else k_wf_shadow<false, false, false, false, false, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
         }
         MT_CUDA_TRY(cudaGetLastError());
         if (timing) MT_TRY(wf_event(timing, iter, 4, st));
