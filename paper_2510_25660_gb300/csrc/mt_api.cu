@@ -1200,7 +1200,9 @@ static mt_status render_common(mt_scene s, mt_film f, int32_t spp, uint64_t seed
     const int kind = mode == 2 ? MT_LAUNCH_BACKWARD : MT_LAUNCH_RENDER;
     const int n_em_smem = (mode == 2 && s->n_em <= 64) ? s->n_em : 0;
     int D;
-    LaunchCfg cfg = warp_tile_cfg(s, kind, f->H, f->W, f->T, spp, n_em_smem * 3, D);
+    // radiance-gradient sums in shared memory: per thread for a few emitters (threads of the configured CTA)
+    const int em_floats = n_em_smem * 3 * (n_em_smem <= MT_EM_PRIVATE ? s->cfg[kind].threads : 1);
+    LaunchCfg cfg = warp_tile_cfg(s, kind, f->H, f->W, f->T, spp, em_floats, D);
     RenderParams p{};
     p.H = f->H;
     p.W = f->W;

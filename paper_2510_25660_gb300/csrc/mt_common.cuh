@@ -446,3 +446,18 @@ __device__ __forceinline__ void splat_add(float *addr, const float *v) {
 #pragma unroll
     for (int k = 0; k < N; ++k) atomicAdd(addr + k, v[k]);
 }
+
+// Sums of the radiance gradients kept per thread in shared memory: entry k (3 per emitter) of thread i at
+// acc[k * blockDim.x + i].  A warp adds up an entry's sums and adds them to global memory once (whole CTA, after a
+// barrier; nothing above MT_EM_PRIVATE emitters).
+#define MT_EM_PRIVATE 4
+__device__ __forceinline__ void em_private_flush(const float *acc, int n_em, float *grad) {
+    if (n_em > MT_EM_PRIVATE) return;
+    const int lane = threadIdx.x & 31;
+    for (int k = threadIdx.x >> 5; k < 3 * n_em; k += blockDim.x >> 5) {
+        float v = 0.f;
+        for (int i = lane; i < (int)blockDim.x; i += 32) v += acc[k * (int)blockDim.x + i];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0 && v != 0.f) atomicAdd(&grad[k], v);
+    }
+}

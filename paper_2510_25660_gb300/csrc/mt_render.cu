@@ -172,7 +172,12 @@ struct Tracer {
                 v.own = v.own + mul(gc, own_r);
             }
             const float3 gr = mul(g, cb);
-            if (p.n_em_smem > 0) {
+            if (p.n_em_smem > 0 && p.n_em_smem <= MT_EM_PRIVATE) {  // this thread's own sums
+                float *a = em_acc + 3 * em * (int)blockDim.x + threadIdx.x;
+                a[0] += gr.x;
+                a[blockDim.x] += gr.y;
+                a[2 * blockDim.x] += gr.z;
+            } else if (p.n_em_smem > 0) {
                 atomicAdd(&em_acc[em * 3], gr.x);
                 atomicAdd(&em_acc[em * 3 + 1], gr.y);
                 atomicAdd(&em_acc[em * 3 + 2], gr.z);
@@ -445,7 +450,8 @@ __global__ void __launch_bounds__(256, MT_MINB_OF(MODE, MEDIA)) k_render(const D
     Counters cnt;
     VRec vrec[MODE == MODE_BWD ? MT_MAX_BWD_DEPTH + 1 : 1];
     if (MODE == MODE_BWD) {
-        for (int i = threadIdx.x; i < p.n_em_smem * 3; i += blockDim.x) em_acc[i] = 0.f;
+        const int n_acc = p.n_em_smem * 3 * (p.n_em_smem <= MT_EM_PRIVATE ? (int)blockDim.x : 1);
+        for (int i = threadIdx.x; i < n_acc; i += blockDim.x) em_acc[i] = 0.f;
         if (threadIdx.x == 0) s_med = 0.f;
         __syncthreads();
     }
@@ -538,8 +544,11 @@ __global__ void __launch_bounds__(256, MT_MINB_OF(MODE, MEDIA)) k_render(const D
     }
     if (MODE == MODE_BWD) {
         __syncthreads();
-        for (int i = threadIdx.x; i < p.n_em_smem * 3; i += blockDim.x)
-            if (em_acc[i] != 0.f) atomicAdd(&p.grad[i], em_acc[i]);
+        if (p.n_em_smem <= MT_EM_PRIVATE)
+            em_private_flush(em_acc, p.n_em_smem, p.grad);
+        else
+            for (int i = threadIdx.x; i < p.n_em_smem * 3; i += blockDim.x)
+                if (em_acc[i] != 0.f) atomicAdd(&p.grad[i], em_acc[i]);
         if (threadIdx.x == 0 && p.gmed && s_med != 0.f) atomicAdd(p.gmed, s_med);
     }
     // counters: one atomic per warp and counter

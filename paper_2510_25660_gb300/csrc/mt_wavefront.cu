@@ -234,10 +234,31 @@ __device__ __forceinline__ float3 wf_grad_at(const WfParams &p, uint32_t pix, fl
     return g;
 }
 
-#define MT_WF_EM_SMEM 64  // emitters whose radiance gradients a CTA sums in shared memory
+// Radiance gradients are summed per CTA in dynamic shared memory.  Up to MT_EM_PRIVATE emitters every thread has sums
+// of its own (entry k of thread i at k * threads + i): float adds of many lanes to one shared word are retried one
+// lane after the other, and sums of fewer terms round less.  Up to MT_WF_EM_SMEM emitters the CTA shares one sum per
+// entry; beyond that the adds go to global memory.
+#define MT_WF_EM_SMEM 64
+extern __shared__ float s_dyn[];
+
+__host__ __device__ __forceinline__ size_t em_smem_bytes(int n_em, int threads) {
+    return n_em <= MT_EM_PRIVATE ? 3 * (size_t)n_em * threads * sizeof(float)
+                                 : (n_em <= MT_WF_EM_SMEM ? 3 * (size_t)n_em * sizeof(float) : 0);
+}
+
+__device__ __forceinline__ void em_grad_init(float *em_acc, int n_em) {
+    const int n = (int)(em_smem_bytes(n_em, blockDim.x) / sizeof(float));
+    for (int k = threadIdx.x; k < n; k += blockDim.x) em_acc[k] = 0.f;
+    __syncthreads();
+}
 
 __device__ __forceinline__ void em_grad_add(const WfParams &p, float *em_acc, int n_em, int em, float3 v) {
-    if (n_em <= MT_WF_EM_SMEM) {
+    if (n_em <= MT_EM_PRIVATE) {
+        float *a = em_acc + 3 * em * (int)blockDim.x + threadIdx.x;
+        a[0] += v.x;
+        a[blockDim.x] += v.y;
+        a[2 * blockDim.x] += v.z;
+    } else if (n_em <= MT_WF_EM_SMEM) {
         atomicAdd(&em_acc[em * 3], v.x);
         atomicAdd(&em_acc[em * 3 + 1], v.y);
         atomicAdd(&em_acc[em * 3 + 2], v.z);
@@ -250,7 +271,8 @@ __device__ __forceinline__ void em_grad_add(const WfParams &p, float *em_acc, in
 
 __device__ __forceinline__ void em_grad_flush(const WfParams &p, const float *em_acc, int n_em) {
     __syncthreads();
-    if (n_em <= MT_WF_EM_SMEM)
+    em_private_flush(em_acc, n_em, p.grad);
+    if (n_em > MT_EM_PRIVATE && n_em <= MT_WF_EM_SMEM)
         for (int k = threadIdx.x; k < n_em * 3; k += blockDim.x)
             if (em_acc[k] != 0.f) atomicAdd(&p.grad[k], em_acc[k]);
 }
@@ -266,13 +288,23 @@ __device__ __forceinline__ void em_grad_flush(const WfParams &p, const float *em
 #ifndef MT_FIN_SMEM_TRIS
 #define MT_FIN_SMEM_TRIS 4096
 #endif
+// Small ones get a copy for each of up to 32 lanes (fin_copies; entry k of copy c at k * copies + c), so that the lanes
+// of a warp do not retry their adds to the same word one after the other.
+__host__ __device__ __forceinline__ int fin_copies(int n_tris) {
+    int c = 32;
+    while (c > 1 && 12 * n_tris * c > 48 * 1024) c >>= 1;
+    return c;
+}
+
 __global__ void __launch_bounds__(256) k_wf_finalize(const DevScene s, const WfParams p) {
-    extern __shared__ float s_galb[];  // [3 n_tris] when n_tris <= MT_FIN_SMEM_TRIS
+    float *s_galb = s_dyn;  // [3 n_tris][copies] when n_tris <= MT_FIN_SMEM_TRIS
     const bool smem = s.n_tris <= MT_FIN_SMEM_TRIS;
+    const int copies = fin_copies(s.n_tris);
     if (smem) {
-        for (int k = threadIdx.x; k < 3 * s.n_tris; k += blockDim.x) s_galb[k] = 0.f;
+        for (int k = threadIdx.x; k < 3 * s.n_tris * copies; k += blockDim.x) s_galb[k] = 0.f;
         __syncthreads();
     }
+    const int mine = threadIdx.x & (copies - 1);
     const uint32_t n = p.counters[C_FIN];
     const uint32_t stride = gridDim.x * blockDim.x;
     const uint32_t n_round = ((n + 31u) / 32u) * 32u;
@@ -291,10 +323,17 @@ __global__ void __launch_bounds__(256) k_wf_finalize(const DevScene s, const WfP
                 const int tri = __float_as_int(a.w);
                 if (tri >= 0) {
                     if (gi.x != 0.f || gi.y != 0.f || gi.z != 0.f) {
-                        float *g = smem ? s_galb + 3 * tri : p.galb + (size_t)tri * 3;
-                        atomicAdd(g, gi.x);
-                        atomicAdd(g + 1, gi.y);
-                        atomicAdd(g + 2, gi.z);
+                        if (smem) {
+                            float *g = s_galb + 3 * tri * copies + mine;
+                            atomicAdd(g, gi.x);
+                            atomicAdd(g + copies, gi.y);
+                            atomicAdd(g + 2 * copies, gi.z);
+                        } else {
+                            float *g = p.galb + (size_t)tri * 3;
+                            atomicAdd(g, gi.x);
+                            atomicAdd(g + 1, gi.y);
+                            atomicAdd(g + 2, gi.z);
+                        }
                     }
                 } else {
                     gm += gi.x + gi.y + gi.z;
@@ -309,8 +348,11 @@ __global__ void __launch_bounds__(256) k_wf_finalize(const DevScene s, const WfP
     if ((threadIdx.x & 31) == 0 && gm != 0.f && p.gmed) atomicAdd(p.gmed, gm);
     if (smem) {  // the CTA's sums, once
         __syncthreads();
-        for (int k = threadIdx.x; k < 3 * s.n_tris; k += blockDim.x)
-            if (s_galb[k] != 0.f) atomicAdd(&p.galb[k], s_galb[k]);
+        for (int k = threadIdx.x; k < 3 * s.n_tris; k += blockDim.x) {
+            float v = 0.f;
+            for (int c = 0; c < copies; ++c) v += s_galb[k * copies + ((c + k) & (copies - 1))];
+            if (v != 0.f) atomicAdd(&p.galb[k], v);
+        }
     }
 }
 
@@ -999,11 +1041,8 @@ __device__ __forceinline__ float3 drad_of(const WfParams &p, int em) {
 template <bool DUMP, bool MEDIA, bool TAN, bool BWD>
 __global__ void __launch_bounds__(256, DUMP || MEDIA || TAN || BWD ? MT_WF_SHADE_MINB : MT_WF_SHADE_FWD_MINB)
     k_wf_shade(const DevScene s, const WfParams p, const uint32_t *qcur, uint32_t *qnext) {
-    __shared__ float em_acc[BWD ? MT_WF_EM_SMEM * 3 : 1];
-    if (BWD) {
-        for (int k = threadIdx.x; k < MT_WF_EM_SMEM * 3; k += blockDim.x) em_acc[k] = 0.f;
-        __syncthreads();
-    }
+    float *em_acc = s_dyn;  // BWD
+    if (BWD) em_grad_init(em_acc, s.n_em);
     const uint32_t n = p.counters[C_CUR];
     uint32_t verts = 0, contribs = 0;
     const uint32_t stride = gridDim.x * blockDim.x;
@@ -1381,11 +1420,8 @@ __device__ __forceinline__ void sh_rays(const DevScene &s, const WfParams &p, ui
 template <bool DUMP, bool CNT, bool WIDE, bool MEDIA, bool BWD, bool FLAT>
 __global__ void __launch_bounds__(256, MT_WF_MINB(MEDIA, FLAT))
     k_wf_shadow(const DevScene s, const WfParams p, int n_idx) {
-    __shared__ float em_acc[BWD ? MT_WF_EM_SMEM * 3 : 1];
-    if (BWD) {
-        for (int k = threadIdx.x; k < MT_WF_EM_SMEM * 3; k += blockDim.x) em_acc[k] = 0.f;
-        __syncthreads();
-    }
+    float *em_acc = s_dyn;  // BWD
+    if (BWD) em_grad_init(em_acc, s.n_em);
     TraceCnt tc{0, 0};
     uint32_t rays = 0, contribs = 0;
     sh_rays<DUMP, CNT, WIDE, MEDIA, BWD, FLAT>(s, p, p.counters[n_idx], em_acc, tc, rays, contribs);
@@ -1570,6 +1606,7 @@ mt_status mt_launch_wavefront(const DevScene &s, const WfParams &p0, int num_sms
         out->used = true;
     }
     const int grid = num_sms * 8;
+    const size_t em_bytes = em_smem_bytes(s.n_em, 256);  // shading and shadow stages of the replay
     // small scenes in a medium: every triangle in turn (not in the counting, wide and dump forms); without a medium the
     // full queues hide the tree's divergence better (Cornell box, 128x128 px, 32 spp: 783 us against 811)
     const bool flat = s.flat != nullptr && s.has_medium;
@@ -1655,8 +1692,8 @@ mt_status mt_launch_wavefront(const DevScene &s, const WfParams &p0, int num_sms
         if (p.mueller) {
             k_wf_shade_pol<<<grid * 2, 128, 0, st>>>(s, p, qa, qb);
         } else if (p.bwd) {
-            if (media) k_wf_shade<false, true, false, true><<<grid, 256, 0, st>>>(s, p, qa, qb);
-            else k_wf_shade<false, false, false, true><<<grid, 256, 0, st>>>(s, p, qa, qb);
+            if (media) k_wf_shade<false, true, false, true><<<grid, 256, em_bytes, st>>>(s, p, qa, qb);
+            else k_wf_shade<false, false, false, true><<<grid, 256, em_bytes, st>>>(s, p, qa, qb);
         } else if (p.sig || p.ps_sig) {  // forward-mode derivative
             if (media) k_wf_shade<false, true, true, false><<<grid, 256, 0, st>>>(s, p, qa, qb);
             else k_wf_shade<false, false, true, false><<<grid, 256, 0, st>>>(s, p, qa, qb);
@@ -1681,14 +1718,14 @@ mt_status mt_launch_wavefront(const DevScene &s, const WfParams &p0, int num_sms
             k_wf_shadow_pol<<<grid, 256, 0, st>>>(s, p);
         } else if (p.bwd) {
             if (media) {
-                if (counters) k_wf_shadow<false, true, false, true, true, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
-                else if (flat) k_wf_shadow<false, false, false, true, true, true><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
-                else k_wf_shadow<false, false, false, true, true, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+                if (counters) k_wf_shadow<false, true, false, true, true, false><<<grid, 256, em_bytes, st>>>(s, p, C_SHADOW);
+                else if (flat) k_wf_shadow<false, false, false, true, true, true><<<grid, 256, em_bytes, st>>>(s, p, C_SHADOW);
+                else k_wf_shadow<false, false, false, true, true, false><<<grid, 256, em_bytes, st>>>(s, p, C_SHADOW);
             } else {
-                if (counters) k_wf_shadow<false, true, false, false, true, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
-                else k_wf_shadow<false, false, false, false, true, false><<<grid, 256, 0, st>>>(s, p, C_SHADOW);
+                if (counters) k_wf_shadow<false, true, false, false, true, false><<<grid, 256, em_bytes, st>>>(s, p, C_SHADOW);
+                else k_wf_shadow<false, false, false, false, true, false><<<grid, 256, em_bytes, st>>>(s, p, C_SHADOW);
             }
-            k_wf_finalize<<<grid, 256, s.n_tris <= MT_FIN_SMEM_TRIS ? 3 * (size_t)s.n_tris * sizeof(float) : 0, st>>>(s, p);
+            k_wf_finalize<<<grid, 256, s.n_tris <= MT_FIN_SMEM_TRIS ? 3 * (size_t)s.n_tris * fin_copies(s.n_tris) * sizeof(float) : 0, st>>>(s, p);
             *launches += 1;
         } else if (dyn) {
             if (counters) k_wf_trace_dyn<true, true><<<grid, 256, 0, st>>>(s, p, qa);
