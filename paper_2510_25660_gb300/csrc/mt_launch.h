@@ -141,7 +141,7 @@ struct WfParams {
     const float *dalb, *drad;
     float dmed;
     // path replay (backward): vertex records [vertex][slot] (a: ratio of the continuation + triangle bits,
-    // b: sum of g * C of contributions made at the vertex, c: own next-event term), the queue of paths
+    // b: sum of g * C of contributions made at the vertex + 1 where c is set, c: own next-event term), the queue of paths
     // that ended in this iteration, gradient inputs and outputs
     int32_t bwd;
     float4 *rec_a, *rec_b, *rec_c;

@@ -316,29 +316,44 @@ __global__ void __launch_bounds__(256) k_wf_finalize(const DevScene s, const WfP
             slot = p.fin_q[q];
             const int end = (int)p.meta[slot].w;
             float3 P = f3(0.f, 0.f, 0.f);
-            for (int i = end; i >= 1; --i) {
-                const size_t r = (size_t)i * p.P + slot;
-                const float4 a = p.rec_a[r], b = p.rec_b[r], c = p.rec_c[r];
-                const float3 gi = mul(P, xyz(a)) + xyz(c);
-                const int tri = __float_as_int(a.w);
-                if (tri >= 0) {
-                    if (gi.x != 0.f || gi.y != 0.f || gi.z != 0.f) {
-                        if (smem) {
-                            float *g = s_galb + 3 * tri * copies + mine;
-                            atomicAdd(g, gi.x);
-                            atomicAdd(g + copies, gi.y);
-                            atomicAdd(g + 2 * copies, gi.z);
-                        } else {
-                            float *g = p.galb + (size_t)tri * 3;
-                            atomicAdd(g, gi.x);
-                            atomicAdd(g + 1, gi.y);
-                            atomicAdd(g + 2, gi.z);
-                        }
-                    }
-                } else {
-                    gm += gi.x + gi.y + gi.z;
+            // four vertices' records are loaded before the first is used: the stage waits on these scattered loads
+            // (b.w = 0: no next-event term was added, rec_c is not set)
+            for (int i0 = end; i0 >= 1; i0 -= 4) {
+                float4 a4[4], b4[4], c4[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (i0 - q < 1) break;
+                    const size_t r = (size_t)(i0 - q) * p.P + slot;
+                    a4[q] = p.rec_a[r];
+                    b4[q] = p.rec_b[r];
+                    c4[q] = p.rec_c[r];
                 }
-                P = P + xyz(b);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (i0 - q < 1) break;
+                    const float4 a = a4[q], b = b4[q];
+                    const float3 own = b.w != 0.f ? xyz(c4[q]) : f3(0.f, 0.f, 0.f);
+                    const float3 gi = mul(P, xyz(a)) + own;
+                    const int tri = __float_as_int(a.w);
+                    if (tri >= 0) {
+                        if (gi.x != 0.f || gi.y != 0.f || gi.z != 0.f) {
+                            if (smem) {
+                                float *g = s_galb + 3 * tri * copies + mine;
+                                atomicAdd(g, gi.x);
+                                atomicAdd(g + copies, gi.y);
+                                atomicAdd(g + 2 * copies, gi.z);
+                            } else {
+                                float *g = p.galb + (size_t)tri * 3;
+                                atomicAdd(g, gi.x);
+                                atomicAdd(g + 1, gi.y);
+                                atomicAdd(g + 2, gi.z);
+                            }
+                        }
+                    } else {
+                        gm += gi.x + gi.y + gi.z;
+                    }
+                    P = P + xyz(b);
+                }
             }
         }
         const uint32_t fs = wf_append(&p.counters[C_FREE], valid);
@@ -1294,8 +1309,7 @@ __global__ void __launch_bounds__(256, DUMP || MEDIA || TAN || BWD ? MT_WF_SHADE
             // the record of this vertex (the shadow stage adds its next-event term)
             const size_t r = (size_t)m.z * p.P + slot;
             p.rec_a[r] = make_float4(rv.x, rv.y, rv.z, __int_as_float(rtri));
-            p.rec_b[r] = make_float4(Sv.x, Sv.y, Sv.z, 0.f);
-            p.rec_c[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+            p.rec_b[r] = make_float4(Sv.x, Sv.y, Sv.z, 0.f);  // w: set with rec_c
         }
         uint32_t qs, ss, fs = 0;
         if (BWD || !qord) {  // the slot of a finished path returns to the free stack (replay: to the finalize queue)
@@ -1397,10 +1411,10 @@ __device__ __forceinline__ void sh_rays(const DevScene &s, const WfParams &p, ui
                     const float3 g = wf_grad_at(p, pix, d.w);
                     const float3 gc = mul(g, cc);
                     const size_t r = (size_t)m.y * p.P + m.w;
-                    const float4 b = p.rec_b[r], c2 = p.rec_c[r];
+                    const float4 b = p.rec_b[r];  // a vertex has one next-event ray
                     const float3 own = mul(gc, xyz(p.sh_cb[i]));
-                    p.rec_b[r] = make_float4(b.x + gc.x, b.y + gc.y, b.z + gc.z, b.w);
-                    p.rec_c[r] = make_float4(c2.x + own.x, c2.y + own.y, c2.z + own.z, c2.w);
+                    p.rec_b[r] = make_float4(b.x + gc.x, b.y + gc.y, b.z + gc.z, 1.f);
+                    p.rec_c[r] = make_float4(own.x, own.y, own.z, 0.f);
                     em_grad_add(p, em_acc, s.n_em, (int)m.z, mul(g, cv));
                     contribs++;
                 } else if (keep) {
