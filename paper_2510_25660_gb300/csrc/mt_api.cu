@@ -496,6 +496,9 @@ static mt_status scene_create_impl(const float *tris, int64_t n, const mt_materi
     sc->n_tris = n;
     sc->n_em = n_em;
     auto &al = sc->al;
+    // one allocation for what scene creation keeps besides the trees (a cudaMalloc and its cudaFree take some 30 us
+    // each): triangles, two material copies, light-unit and leaf indices, shading records, and room for the small ones
+    MT_TRY(al.reserve((size_t)n * (9 * 4 + sizeof(mt_material) + 16 + 4 + 4 + 32) + 64 * 256, "scene"));
     float *d_tris;
     mt_material *d_mats;
     mt_emitter *d_em;
@@ -519,7 +522,13 @@ static mt_status scene_create_impl(const float *tris, int64_t n, const mt_materi
             return MT_ERR_INVALID_ARGUMENT;
         }
     }
-    MT_TRY(mt_build_bvh(d_tris, (int32_t)n, st, al, &sc->bvh));
+    {  // the trees get allocations of their own
+        const size_t left = al.arena_left;
+        al.arena_left = 0;
+        const mt_status bs = mt_build_bvh(d_tris, (int32_t)n, st, al, &sc->bvh);
+        al.arena_left = left;
+        MT_TRY(bs);
+    }
     DevScene &D = sc->dev;
     D.nodes = sc->bvh.nodes;
     D.wnodes = sc->bvh.wnodes;
@@ -664,6 +673,7 @@ static mt_status scene_create_impl(const float *tris, int64_t n, const mt_materi
     D.tan_half = hcam.tan_half;
     D.err = sc->err;
     D.counters = sc->counters;
+    al.arena_left = 0;  // later allocations are their own
     for (int k = 0; k < 4; ++k) sc->cfg[k] = LaunchCfg{256, 0, 0, sc->num_sms, 0, -1, 0};
     // renders and backward passes add to the film in L2 instead of privatising it: zeroing and writing a
     // warp's histograms costs more than the few adds of its paths, and the shared memory costs resident

@@ -1255,13 +1255,12 @@ mt_status mt_build_bvh(const float *d_tris, int32_t n, cudaStream_t st, mt::Allo
         MT_CUDA_TRY(cudaMemsetAsync(counters + 1, 0, sizeof(int), st));
         k_children<<<(nt + 127) / 128, 128, 0, st>>>(taskA, nt, decs, nodes, counters, taskB, small);
         MT_CUDA_TRY(cudaGetLastError());
+        // the counters and every task the level can have made, behind one wait
+        large.resize(std::min(2 * nt, max_tasks));
         MT_CUDA_TRY(cudaMemcpyAsync(hc, counters, sizeof(hc), cudaMemcpyDeviceToHost, st));
+        MT_CUDA_TRY(cudaMemcpyAsync(large.data(), taskB, large.size() * sizeof(Task), cudaMemcpyDeviceToHost, st));
         MT_CUDA_TRY(cudaStreamSynchronize(st));
-        large.resize(hc[1]);
-        if (hc[1] > 0) {
-            MT_CUDA_TRY(cudaMemcpyAsync(large.data(), taskB, hc[1] * sizeof(Task), cudaMemcpyDeviceToHost, st));
-            MT_CUDA_TRY(cudaStreamSynchronize(st));
-        }
+        large.resize(std::min<size_t>(large.size(), (size_t)hc[1]));
     }
     if (hc[2] > 0) {
         BNode *loc;

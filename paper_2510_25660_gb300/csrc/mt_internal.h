@@ -26,14 +26,36 @@ mt_status alloc_device(void **p, size_t bytes, const char *what);
 // freed memory for reuse), for temporaries used on one stream only
 mt_status alloc_device_async(void **p, size_t bytes, const char *what, cudaStream_t st);
 
+#define MT_ALLOC_TRY(call)               \
+    do {                                 \
+        const mt_status s_ = (call);     \
+        if (s_ != MT_OK) return s_;      \
+    } while (0)
+
 struct AllocList {
     std::vector<void *> ptrs;
     bool stream_ordered = false;  // allocate and free on `stream` (temporaries)
     cudaStream_t stream = nullptr;
+    // the rest of one larger allocation that later ones are cut from (256-byte steps) while they fit
+    char *arena = nullptr;
+    size_t arena_left = 0;
+    mt_status reserve(size_t bytes, const char *what) {
+        arena_left = 0;
+        MT_ALLOC_TRY(alloc(&arena, bytes, what));
+        arena_left = bytes;
+        return MT_OK;
+    }
     template <class T>
     mt_status alloc(T **p, size_t count, const char *what) {
         void *q = nullptr;
         const size_t bytes = count * sizeof(T) + (count == 0 ? 16 : 0);
+        const size_t step = (bytes + 255) & ~(size_t)255;
+        if (step <= arena_left) {
+            *p = (T *)arena;
+            arena += step;
+            arena_left -= step;
+            return MT_OK;
+        }
         mt_status st = stream_ordered ? alloc_device_async(&q, bytes, what, stream) : alloc_device(&q, bytes, what);
         if (st != MT_OK) return st;
         ptrs.push_back(q);
@@ -46,6 +68,7 @@ struct AllocList {
             else cudaFree(p);
         }
         ptrs.clear();
+        arena_left = 0;
     }
     size_t bytes = 0;
 };
