@@ -591,10 +591,10 @@ static mt_status scene_create_impl(const float *tris, int64_t n, const mt_materi
     // cost) is long for so few triangles.  Frames of 128x128 px, 32 spp, depth 6, tree / loop in the persistent form:
     // in a medium, closed rooms and boxes of 13 to 37 triangles 1022 / 890 to 2325 / 1457 us, random open meshes of 6,
     // 16, 36, 48, 64 triangles 917 / 741, 1174 / 881, 1436 / 1290, 1476 / 1484, 1560 / 1710, but planes of 2 to 6
-    // triangles 697 / 977 to 1623 / 1828; without one, 20-triangle sphere (SAH cost 13.6) 891 / 471, 37-triangle room
-    // (14.1) 601 / 598, Cornell box (14.5) 611 / 596, 25-triangle room (10.2) 439 / 493, 36 random triangles (5.0) 188 /
+    // triangles 697 / 977 to 1623 / 1828; without one, 20-triangle sphere (SAH cost 12.9) 891 / 471, 37-triangle room
+    // (14.1) 601 / 598, Cornell box (14.3) 611 / 596, 25-triangle room (10.2) 439 / 493, 36 random triangles (5.0) 188 /
     // 242.  Small frames gain more: Cornell box 64x64, 16 spp 135 / 100.
-    if (n >= 8 && n <= 48 && (med || sc->bvh.sah >= 13.0)) {
+    if (n >= 8 && n <= 48 && (med || sc->bvh.sah >= 12.5)) {
         float4 *flat;
         MT_TRY(al.alloc(&flat, (size_t)6 * ((n + 1) / 2), "triangle pairs"));
         uint4 *box;

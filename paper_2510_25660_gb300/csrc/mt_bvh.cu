@@ -28,12 +28,14 @@
 namespace {
 
 constexpr int NB = 32;          // bins per axis
-// SAH cost of one traversal step relative to one triangle test (leaf decision).
-// A triangle test (48-byte record, watertight test) costs more than a node test
-// on GB300: 0.5 measured 96.8 ms against 97.6 ms at 1.0 and 107-109 ms at 2-3
-// for the 512x512x256-spp forward render of the 1.16M-triangle scene.
+// SAH cost of one traversal step relative to one triangle test (leaf decision):
+// a node test and a triangle test (48-byte record in the ray's axis order) take
+// about the same instructions.  512x512x256-spp render of the 1.16M-triangle
+// scene 61.6 / 61.5 / 61.35 / 61.3 / 62.0 ms at 0.35 / 0.5 / 0.75 / 1 / 1.5,
+// exhaustive NLOS scan 10.97 / 10.94 / 10.76 / 10.74 / 10.86 ms, and the build is
+// shorter: loading the scene 7.82 / 7.75 / 7.50 / 7.35 / 7.08 ms.
 #ifndef MT_SAH_CT
-#define MT_SAH_CT 0.5f
+#define MT_SAH_CT 1.0f
 #endif
 // The tree does not depend on this threshold (the same binned SAH decisions are
 // taken either way); a CTA steps through its subtree node by node, so smaller
