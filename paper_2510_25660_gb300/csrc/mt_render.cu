@@ -385,12 +385,11 @@ struct Tracer {
         cnt.vertices++;
         const float3 x = ps.o + ps.d * th;
         if (!(ps.depth == 1 && (p.flags & MT_UNWARP))) ps.opl += th;
-        float3 v0, v1, v2;
-        tri_vertices(s, k, v0, v1, v2);
-        const float3 ng = normalize(cross(v1 - v0, v2 - v0));
+        const float4 sn = __ldg(&s.shrec[2 * (size_t)k]);  // normal + light unit
+        const float3 ng = xyz(sn);
         const float3 wo = -ps.d;
         const float cwo = dot(ng, wo);
-        const int unit = __ldg(&s.tri_unit[orig]);
+        const int unit = __float_as_int(sn.w);
         // the vertex is recorded before anything can end the path here, so that light
         // found at the last vertex still reaches the earlier vertices' gradients
         if (MODE == MODE_BWD) vr[ps.depth].tri = orig;
@@ -413,7 +412,7 @@ struct Tracer {
         float3 tb, bb;
         onb(n, tb, bb);
         const float3 wol = to_local(wo, tb, bb, n);
-        const float4 mm = __ldg(&s.mats[orig]);
+        const float4 mm = __ldg(&s.shrec[2 * (size_t)k + 1]);
         const Mat m{xyz(mm), mm.w};
         if (MODE == MODE_TAN)
             ps.dv = p.dalb ? f3(p.dalb[orig * 3], p.dalb[orig * 3 + 1], p.dalb[orig * 3 + 2]) : f3(0.f, 0.f, 0.f);
