@@ -174,7 +174,8 @@ mt_status mt_film_set_window(mt_film film, int32_t frame_H, int32_t row0);
  * scene that needs a larger pool than the scene holds (a render of more paths,
  * up to the pool size of mt_set_wavefront_pool), waits every few iterations
  * until `stream` has finished the iteration two back (the host stays ahead of
- * the GPU; nothing is copied for it), and refuses to run under stream capture
+ * the GPU; nothing is copied for it; a render whose paths all fit the pool waits
+ * once, for its last iteration), and refuses to run under stream capture
  * when it would allocate (INVALID_ARGUMENT).  Errors: INVALID_ARGUMENT (spp < 1,
  * max_depth outside [1, 64], film C != 3), OUT_OF_MEMORY (path pool), CUDA. */
 mt_status mt_render(mt_scene scene, mt_film film, int32_t spp, uint64_t seed, int32_t max_depth,

