@@ -120,7 +120,7 @@ struct mt_scene_s {
     float4 *ysamp = nullptr;
     int32_t *ysamp_tri = nullptr;
     long long ysamp_cap = 0;
-    int32_t *sorder = nullptr;  // sensor order of exhaustive grids
+    int32_t *sorder = nullptr;  // sensor order of exhaustive grids, 2 sorder_cap entries
     int32_t sorder_cap = 0;
     GraphCache nlos_graph;
     cudaStream_t cap_stream = nullptr;  // private stream the NLOS graph is captured on
@@ -1559,7 +1559,7 @@ static mt_status nlos_prepare(mt_scene s, mt_film f, const mt_scan *sc, int32_t 
             MT_CUDA_TRY(cudaStreamIsCapturing(st, &cs));
             int32_t *order = nullptr;
             if (cs == cudaStreamCaptureStatusNone &&
-                s->al.alloc(&order, (size_t)sc->n_sensors, "nlos sensor order") == MT_OK) {
+                s->al.alloc(&order, 2 * (size_t)sc->n_sensors, "nlos sensor order") == MT_OK) {
                 s->sorder = order;
                 s->sorder_cap = sc->n_sensors;
             }

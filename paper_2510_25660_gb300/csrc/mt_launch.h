@@ -64,7 +64,7 @@ struct NlosParams {
     // the default forms (no privatised bins, no aggregation, the automatic tile); not used by the dump
     int32_t scan;              // 1: k_nlos_scan
     int32_t run;               // hidden samples per warp item of k_nlos_pairs (0: k_nlos)
-    const int32_t *order;      // scratch for k_nlos_pairs' sensor order (null: as given)
+    const int32_t *order;      // scratch of 2 n_s for k_nlos_pairs' sensor order (null: as given)
 };
 
 // Path pool layout of the wavefront form.  MT_WF_AOS = 1: one 128-byte record

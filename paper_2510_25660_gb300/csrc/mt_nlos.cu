@@ -260,7 +260,8 @@ __global__ void __launch_bounds__(256) k_nlos_ysample_ordered(const DevScene s, 
 // Sensor order of k_nlos_pairs: by the Morton code of their position on the wall (32 x 32 cells over the points'
 // extent along two axes across the wall normal), so that the 32 rays of a warp go from one point y to a patch of the
 // wall instead of a line across it (16x16 x 32x32 pairs, 1024 samples: 14.8 -> 10.97 ms).  One CTA; the order within
-// a cell is free.
+// a cell is free.  A sensor's cell is computed once and kept behind the order (order holds 2 n_s entries): counted and
+// placed from one value, the order is a permutation of the sensors whatever the rounding of the cell, NaN included.
 __global__ void __launch_bounds__(1024) k_nlos_sensor_order(const NlosParams p, int32_t *order) {
     __shared__ int s_box[4];  // ordered ints: lower t, b; upper t, b
     __shared__ uint32_t s_cnt[1024], s_warp[32];
@@ -285,15 +286,16 @@ __global__ void __launch_bounds__(1024) k_nlos_sensor_order(const NlosParams p, 
     __syncthreads();
     const float lo_u = o2f(s_box[0]), lo_v = o2f(s_box[1]);
     const float ext = fmaxf(fmaxf(o2f(s_box[2]) - lo_u, o2f(s_box[3]) - lo_v), 1e-30f);
-    auto cell = [&](int i) {
+    int32_t *cell = order + p.n_s;
+    for (int i = threadIdx.x; i < p.n_s; i += blockDim.x) {
         const float3 x = f3(p.sensors[3 * i], p.sensors[3 * i + 1], p.sensors[3 * i + 2]);
         const int cu = min(max((int)((dot(x, tb) - lo_u) / ext * 32.0f), 0), 31);
         const int cv = min(max((int)((dot(x, bb) - lo_v) / ext * 32.0f), 0), 31);
         uint32_t m = 0;
         for (int k = 0; k < 5; ++k) m |= ((uint32_t)(cu >> k & 1) << (2 * k)) | ((uint32_t)(cv >> k & 1) << (2 * k + 1));
-        return m;
-    };
-    for (int i = threadIdx.x; i < p.n_s; i += blockDim.x) atomicAdd(&s_cnt[cell(i)], 1u);
+        cell[i] = (int)m;
+        atomicAdd(&s_cnt[m], 1u);
+    }
     __syncthreads();
     // exclusive scan of the 1024 counts
     const uint32_t c = s_cnt[threadIdx.x];
@@ -316,7 +318,7 @@ __global__ void __launch_bounds__(1024) k_nlos_sensor_order(const NlosParams p, 
     __syncthreads();
     s_cnt[threadIdx.x] = x - c + (w > 0 ? s_warp[w - 1] : 0u);
     __syncthreads();
-    for (int i = threadIdx.x; i < p.n_s; i += blockDim.x) order[atomicAdd(&s_cnt[cell(i)], 1u)] = i;
+    for (int i = threadIdx.x; i < p.n_s; i += blockDim.x) order[atomicAdd(&s_cnt[cell[i]], 1u)] = i;
 }
 
 // exhaustive grid: a warp takes 32 sensors of a laser, one per lane, and a run of p.run of its hidden
