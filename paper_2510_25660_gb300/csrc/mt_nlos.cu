@@ -49,6 +49,39 @@ __device__ __forceinline__ int pick_hidden(const NlosParams &p, uint32_t u) {
     return p.hidden_first + lo;
 }
 
+// The arithmetic of a connection is spelled out, once for all kernels of this file: which product of a sum of
+// products is fused is the compiler's choice at each place a function is inlined, and a path length that differs in
+// its last bit moves a connection across a bin edge (about 75 of the 67 M that reach the film of 16x16 x 32x32 pairs,
+// T = 4096, 1024 samples: 3e-4 to 4e-3 of the film's norm, while each kernel repeats its own film to 1e-8).  Each sum
+// has one order; dot_xyz and dot_yxz name the order in which the products enter.
+__device__ __forceinline__ float dot_xyz(float3 a, float3 b) {
+    return fmaf(a.z, b.z, fmaf(a.y, b.y, __fmul_rn(a.x, b.x)));
+}
+__device__ __forceinline__ float dot_yxz(float3 a, float3 b) {
+    return fmaf(a.z, b.z, fmaf(a.x, b.x, __fmul_rn(a.y, b.y)));
+}
+
+// uniform point on a triangle (tri_point)
+__device__ __forceinline__ float3 hidden_point(float3 v0, float3 v1, float3 v2, float u1, float u2) {
+    const float su = sqrtf(u1);
+    const float b0 = 1.0f - su, b1 = __fmul_rn(u2, su), b2 = __fsub_rn(1.0f - b0, b1);
+    auto mix = [&](float x0, float x1, float x2) { return fmaf(x2, b2, fmaf(x0, b0, __fmul_rn(x1, b1))); };
+    return f3(mix(v0.x, v1.x, v2.x), mix(v0.y, v1.y, v2.y), mix(v0.z, v1.z, v2.z));
+}
+
+__device__ __forceinline__ float3 hidden_normal(float3 v0, float3 v1, float3 v2) {
+    const float3 a = v1 - v0, b = v2 - v0;
+    auto minor = [](float x, float y, float z, float w) { return fmaf(x, y, -__fmul_rn(z, w)); };
+    const float3 c = f3(minor(a.y, b.z, a.z, b.y), minor(a.z, b.x, a.x, b.z), minor(a.x, b.y, a.y, b.x));
+    return c * (1.0f / sqrtf(dot_yxz(c, c)));
+}
+
+// p moved off its surface along the unit normal n
+__device__ __forceinline__ float3 lift(float3 p, float3 n) {
+    const float e = eps_of(p);
+    return f3(fmaf(n.x, e, p.x), fmaf(n.y, e, p.y), fmaf(n.z, e, p.z));
+}
+
 struct HiddenSample {
     float3 y, ny;
     float d1, partial;  // partial = fw cos_l fh cos_y1 / d1^2 * A (0 if invalid or occluded)
@@ -64,22 +97,22 @@ __device__ __forceinline__ HiddenSample sample_on(const DevScene &s, const NlosP
     float3 v0, v1, v2;
     tri_vertices(s, k, v0, v1, v2);
     h.tri = tri;
-    h.y = tri_point(v0, v1, v2, u24(R.y), u24(R.z));
+    h.y = hidden_point(v0, v1, v2, u24(R.y), u24(R.z));
     h.partial = 0.f;
     h.cl = h.cy1 = 0.f;
-    const float3 ng = normalize(cross(v1 - v0, v2 - v0));
+    const float3 ng = hidden_normal(v0, v1, v2);
     const float3 d1v = h.y - xl;
-    h.d1 = sqrtf(dot(d1v, d1v));
+    h.d1 = sqrtf(dot_yxz(d1v, d1v));
     if (!(h.d1 > 0.f)) return h;
     const float3 w1 = d1v * (1.0f / h.d1);
-    h.ny = dot(ng, -w1) >= 0.f ? ng : -ng;
-    const float cl = dot(p.nw, w1), cy1 = -dot(h.ny, w1);
+    h.ny = dot_yxz(ng, -w1) >= 0.f ? ng : -ng;
+    const float cl = dot_yxz(p.nw, w1), cy1 = -dot_yxz(h.ny, w1);
     h.cl = cl;
     h.cy1 = cy1;
     if (!(cl > 0.f && cy1 > 0.f)) return h;
-    const float3 xlo = xl + p.nw * eps_of(xl);
+    const float3 xlo = lift(xl, p.nw);
     const float3 r1 = h.y - xlo;
-    const float l1 = sqrtf(dot(r1, r1));
+    const float l1 = sqrtf(dot_yxz(r1, r1));
     rays++;
     const RayT ray = make_ray(s, xlo, r1 * (1.0f / l1));
     if (trace_any<CNT>(s, ray, l1 - eps_of(h.y), tc)) return h;
@@ -88,6 +121,34 @@ __device__ __forceinline__ HiddenSample sample_on(const DevScene &s, const NlosP
     const float area = p.hidden_area_dev ? __ldg(p.hidden_area_dev) : p.hidden_area;
     h.partial = p.fw * cl * fh * cy1 / (h.d1 * h.d1) * area;
     return h;
+}
+
+// confocal connection of a visible hidden sample (x_s = x_l, the same segment both ways)
+__device__ __forceinline__ float confocal_value(const NlosParams &p, const HiddenSample &h) {
+    return h.partial * h.cy1 * h.cl * p.fw / (h.d1 * h.d1);
+}
+
+// connection of a hidden sample of its laser (ya = y, d1; yb = normal, partial) with the sensor at xs: its value (0:
+// none) and its path length
+template <bool CNT>
+__device__ __forceinline__ float sensor_value(const DevScene &s, const NlosParams &p, float4 ya, float4 yb, float3 xs,
+                                              float &opl, TraceCnt &tc, uint32_t &rays) {
+    if (!(yb.w > 0.f)) return 0.f;
+    const float3 y = xyz(ya), ny = xyz(yb);
+    const float3 d2v = xs - y;
+    const float d2 = sqrtf(dot_xyz(d2v, d2v));
+    if (!(d2 > 0.f)) return 0.f;
+    const float3 w2 = d2v * (1.0f / d2);
+    const float cs = -dot_yxz(p.nw, w2), cy2 = dot_yxz(ny, w2);
+    if (!(cs > 0.f && cy2 > 0.f)) return 0.f;
+    const float3 yo = lift(y, ny);
+    const float3 r2 = xs - yo;
+    const float l2 = sqrtf(dot_xyz(r2, r2));
+    rays++;
+    const RayT ray = make_ray(s, yo, r2 * (1.0f / l2));
+    if (trace_any<CNT>(s, ray, l2 - eps_of(xs), tc)) return 0.f;
+    opl = ya.w + d2;
+    return yb.w * cy2 * cs * p.fw / (d2 * d2);
 }
 
 __device__ __forceinline__ uint4 hidden_words(const NlosParams &p, int l, uint32_t smp) {
@@ -192,8 +253,8 @@ __global__ void __launch_bounds__(256, MT_NLOS_SCAN_MINB) k_nlos_scan(const DevS
                 conns++;
                 const uint4 R = hidden_words(p, row, p.sample_offset + (uint32_t)(j0 + j));
                 const HiddenSample h = sample_on<CNT>(s, p, R, tri, __ldg(&s.leaf_of[tri]), xl, tc, rays);
-                if (h.partial > 0.f) {  // confocal: x_s = x_l, the same segment both ways
-                    const float H = h.partial * h.cy1 * h.cl * p.fw / (h.d1 * h.d1);
+                if (h.partial > 0.f) {
+                    const float H = confocal_value(p, h);
                     if (H > 0.f) {
                         contribs++;
                         const float v = H * p.scale;
@@ -349,25 +410,12 @@ __global__ void __launch_bounds__(256, MT_NLOS_PAIRS_MINB) k_nlos_pairs(const De
         for (int j = j0; j < j1; ++j) {
             const float4 ya = __ldg(&p.ysamp[2 * ((size_t)l * p.spp + j)]), yb = __ldg(&p.ysamp[2 * ((size_t)l * p.spp + j) + 1]);
             conns++;
-            if (!(yb.w > 0.f)) continue;
-            const float3 y = xyz(ya), ny = xyz(yb);
-            const float3 d2v = xs - y;
-            const float d2 = sqrtf(dot(d2v, d2v));
-            if (!(d2 > 0.f)) continue;
-            const float3 w2 = d2v * (1.0f / d2);
-            const float cs = -dot(p.nw, w2), cy2 = dot(ny, w2);
-            if (!(cs > 0.f && cy2 > 0.f)) continue;
-            const float3 yo = y + ny * eps_of(y);
-            const float3 r2 = xs - yo;
-            const float l2 = sqrtf(dot(r2, r2));
-            rays++;
-            const RayT ray = make_ray(s, yo, r2 * (1.0f / l2));
-            if (trace_any<CNT>(s, ray, l2 - eps_of(xs), tc)) continue;
-            const float H = yb.w * cy2 * cs * p.fw / (d2 * d2);
+            float opl = 0.f;
+            const float H = sensor_value<CNT>(s, p, ya, yb, xs, opl, tc, rays);
             if (H > 0.f) {
                 contribs++;
                 const float v = H * p.scale;
-                nlos_splat(p, row, ya.w + d2, v);
+                nlos_splat(p, row, opl, v);
                 steady += v;
             }
         }
@@ -424,36 +472,15 @@ __global__ void __launch_bounds__(256) k_nlos(const DevScene s, const NlosParams
                 const HiddenSample h = sample_hidden<CNT>(s, p, li, smp, xl, tc, rays);
                 tri = h.tri;
                 if (h.partial > 0.f) {
-                    // confocal: x_s = x_l, the same segment both ways
-                    H = h.partial * h.cy1 * h.cl * p.fw / (h.d1 * h.d1);
+                    H = confocal_value(p, h);
                     opl = 2.0f * h.d1;
                 }
             } else {
                 const int si = s0 + r;
                 const float3 xs = f3(p.sensors[3 * si], p.sensors[3 * si + 1], p.sensors[3 * si + 2]);
                 const size_t yi = (size_t)l * p.spp + sj;
-                const float4 ya = p.ysamp[2 * yi], yb = p.ysamp[2 * yi + 1];
                 tri = DUMP ? p.ysamp_tri[yi] : -1;
-                if (yb.w > 0.f) {
-                    const float3 y = xyz(ya), ny = xyz(yb);
-                    const float3 d2v = xs - y;
-                    const float d2 = sqrtf(dot(d2v, d2v));
-                    if (d2 > 0.f) {
-                        const float3 w2 = d2v * (1.0f / d2);
-                        const float cs = -dot(p.nw, w2), cy2 = dot(ny, w2);
-                        if (cs > 0.f && cy2 > 0.f) {
-                            const float3 yo = y + ny * eps_of(y);
-                            const float3 r2 = xs - yo;
-                            const float l2 = sqrtf(dot(r2, r2));
-                            rays++;
-                            const RayT ray = make_ray(s, yo, r2 * (1.0f / l2));
-                            if (!trace_any<CNT>(s, ray, l2 - eps_of(xs), tc)) {
-                                H = yb.w * cy2 * cs * p.fw / (d2 * d2);
-                                opl = ya.w + d2;
-                            }
-                        }
-                    }
-                }
+                H = sensor_value<CNT>(s, p, p.ysamp[2 * yi], p.ysamp[2 * yi + 1], xs, opl, tc, rays);
             }
             if (H > 0.f) {
                 contribs++;
