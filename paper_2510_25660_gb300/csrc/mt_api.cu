@@ -1451,6 +1451,22 @@ static mt_status hidden_table(mt_scene s, int first, int n, uint32_t *cdf, uint3
     return MT_OK;
 }
 
+// Exhaustive grids for which k_nlos, which gives every lane a pair, is faster than k_nlos_pairs (lasers x sensors x
+// samples: k_nlos_pairs / k_nlos in us).
+// - Small grids of few samples: a warp's run of samples is a chain of traversals that nothing hides. 1x31x4 59 / 40,
+//   16x31x4 115 / 75, 32x256x6 137 / 96, 16x1024x8 147 / 109.
+// - Sensors that fill less than half of a warp, once the lasers (one CTA each) fill the GPU: 32 lasers per sensor, 64
+//   for long captures, whose samples k_nlos_pairs spreads over more warps, none for short ones. 608x1x1024 1066 / 439,
+//   608x4x1024 1296 / 744, 608x16x1024 1732 / 1383 (608x19x1024 1772 / 1660, 2000x19x1024 4255 / 4590); 32x1x1024 261 /
+//   200, 64x2x2048 403 / 449, 152x4x2048 764 / 768, 304x8x1024 825 / 744, 100x12x1024 458 / 711; 100x1x8192 1276 /
+//   1087, 64x1x32768 2696 / 3582, 304x2x32768 12668 / 8738; 304x1x4 99 / 90, 8x16x4 122 / 97, 608x16x32 195 / 164; one
+//   sensor leaves 31 lanes idle: 1x1x1024 198 / 165, 16x1x1024 246 / 199.
+static bool pairs_idle(long long n_lasers, long long n_sensors, long long spp) {
+    if (spp <= 12 && n_lasers * n_sensors * spp < 1 << 18) return true;
+    if (n_sensors == 1 && spp <= 1024) return true;
+    return n_sensors <= 16 && n_lasers >= (spp <= 32 ? 0 : spp <= 4096 ? 32 : 64) * n_sensors;
+}
+
 // Launch parameters of an NLOS capture over the given sampling table and scratch
 // (area_dev: device copy of the hidden area read by the kernels, or null to use
 // `area`); shared by the allocating and the allocation-free entry points.
@@ -1499,7 +1515,7 @@ static void nlos_fill(mt_scene s, mt_film f, const mt_scan *sc, int32_t spp, uin
     p.scan = plain && !exh && spp >= MT_NLOS_ORDER_SPP && rows * spp >= MT_NLOS_ORDER_TOTAL ? 1 : 0;
     // runs of 128 hidden samples, shorter (down to 4) where that gives fewer than 64 warps per SM
     p.run = 0;
-    if (plain && exh) {
+    if (plain && exh && !pairs_idle(sc->n_lasers, sc->n_sensors, spp)) {
         const long long groups = (long long)sc->n_lasers * ((sc->n_sensors + 31) / 32);
         p.run = (int)std::max<long long>(4, std::min<long long>(128, groups * spp / (64LL * s->num_sms)));
         // the item count must fit the claim counter

@@ -9,9 +9,10 @@
 // per sample.  All scan pairs are one persistent launch.  The default forms add
 // to the film in L2: k_nlos_scan takes a scan point per CTA and its samples in
 // the order of the hidden surface, k_nlos_pairs takes 32 sensors of a laser per
-// warp.  k_nlos (a launch configuration that privatises bins, aggregates or
-// sets a tile, and the dump) pulls tiles of consecutive film rows and keeps the
-// rows' time histograms in shared memory.  In the exhaustive grid the hidden
+// warp.  k_nlos (small exhaustive grids and those of few sensors, a launch
+// configuration that privatises bins, aggregates or sets a tile, and the dump)
+// pulls tiles of consecutive film rows and keeps the rows' time histograms in
+// shared memory.  In the exhaustive grid the hidden
 // samples of a laser are drawn once (visibility x_l -> y included) by
 // k_nlos_ysample and shared by all its sensors.
 #include "mt_common.cuh"
