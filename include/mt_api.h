@@ -329,7 +329,8 @@ mt_status mt_scene_stats(mt_scene scene, int64_t *out);
  *   tile         RENDER/BACKWARD: pixels of one image row owned by one warp at
  *                a time (default: pixels for 32 paths, fewer where the frame
  *                would not fill the GPU); NLOS: scan rows owned by one CTA at
- *                a time (default: 1; EXHAUSTIVE 32)
+ *                a time (default: 1; EXHAUSTIVE 32, with priv_bins other
+ *                than 0 as many as have all their bins in 96 KB)
  *   ctas_per_sm  cap on resident CTAs per SM (0 = occupancy maximum)
  *   priv_bins    time bins per pixel (scan row) accumulated in shared memory
  *                before one write to HBM; later bins are added to the film in

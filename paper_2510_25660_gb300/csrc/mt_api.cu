@@ -924,8 +924,11 @@ static LaunchCfg nlos_cfg(const mt_scene_s *s, int kind, int32_t T, int &D) {
     const size_t budget = (size_t)std::min(s->smem_optin, 220 * 1024) - 1024;
     int tile = c.tile > 0 ? c.tile : 0;
     // automatic: one scan row per CTA (64x64 points, T = 4096, 1024 samples: 1.60 ms with its bins in shared memory,
-    // 1.77 / 2.51 ms for 2 / 4 rows), 32 sensors of a laser
-    if (tile == 0) tile = kind == MT_LAUNCH_NLOS_EXHAUSTIVE ? 32 : 1;
+    // 1.77 / 2.51 ms for 2 / 4 rows).  Exhaustive: 32 sensors of a laser, or as many as have all their bins in 96 KB
+    // where bins are privatised (16 lasers x 1024 sensors, T = 4096, 1 / 4 / 64 samples: 130 / 229 / 473 us with 6
+    // sensors, 192 / 277 / 519 us with 32 and the first 1700 bins).
+    if (tile == 0 && kind != MT_LAUNCH_NLOS_EXHAUSTIVE) tile = 1;
+    if (tile == 0) tile = c.priv == 0 ? 32 : std::max(1, std::min(32, 96 * 1024 / (int)sizeof(float) / std::max(T, 1)));
     const size_t fixed = (size_t)tile * 4 + 64;
     const size_t avail = budget > fixed ? budget - fixed : 0;
     D = (int)std::min<size_t>((size_t)T, avail / ((size_t)tile * 4));
