@@ -294,7 +294,7 @@ def main():
     wavefront = bool(cfg and cfg.get("options", 0) & api.MT_OPT_WAVEFRONT)
     if wavefront:
         # CUDA events at the stage boundaries time the traversal kernels inside the timed region
-        s.set_launch(api.MT_LAUNCH_RENDER, cfg["threads"], cfg["tile"], cfg["ctas_per_sm"], cfg.get("priv", -1),
+        s.set_launch(api.MT_LAUNCH_RENDER, cfg["threads"], cfg["tile"], cfg["ctas_per_sm"], cfg.get("priv", 0),
                      cfg["options"] | api.MT_OPT_STAGE_TIMING)
     film, steady = api.new_film(f.H, f.W, f.T)
     flush = torch.empty(L2_FLUSH_BYTES // 4, dtype=torch.float32, device="cuda")
@@ -598,7 +598,7 @@ def comparisons(api, autotune, scenes, per_point=256):
     sub = pts[:per_point].contiguous()
     ref, ref_s = api.render_nlos(s, sub, None, api.MT_CONFOCAL, T, 0.0, W0, 16 * spp, 99)
     # one plain launch per scan point through the same API, same kernel and launch configuration
-    s.set_launch(api.MT_LAUNCH_NLOS, cfg.get("threads", 0), cfg.get("tile", 0), 0, cfg.get("priv", -1),
+    s.set_launch(api.MT_LAUNCH_NLOS, cfg.get("threads", 0), cfg.get("tile", 0), 0, cfg.get("priv", 0),
                  cfg.get("options", 0) | api.MT_OPT_NO_GRAPH)
     pf = torch.empty((per_point, T), device="cuda")
     ps = torch.empty(per_point, device="cuda")

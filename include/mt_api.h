@@ -320,7 +320,8 @@ mt_status mt_scene_set_pulse(mt_scene scene, uint32_t shape, float a, float b);
 mt_status mt_scene_stats(mt_scene scene, int64_t *out);
 
 /* Launch configuration used by the next launches of this scene (set by the
- * autotuner; 0 keeps a field at its default), per kind: MT_LAUNCH_RENDER,
+ * autotuner; 0 sets a field to its default, so all zeros restore the
+ * configuration of a new scene), per kind: MT_LAUNCH_RENDER,
  * MT_LAUNCH_BACKWARD, MT_LAUNCH_NLOS (scan-point grids) and
  * MT_LAUNCH_NLOS_EXHAUSTIVE (laser x sensor grids, whose scene default is 32
  * sensors per tile with priv_bins = 0: the lanes of a warp take neighbouring
@@ -334,8 +335,8 @@ mt_status mt_scene_stats(mt_scene scene, int64_t *out);
  *   ctas_per_sm  cap on resident CTAs per SM (0 = occupancy maximum)
  *   priv_bins    time bins per pixel (scan row) accumulated in shared memory
  *                before one write to HBM; later bins are added to the film in
- *                global memory directly.  -1 = as many as fit, 0 = none (what
- *                a new scene uses).
+ *                global memory directly.  -1 = as many as fit, 0 = none (the
+ *                default of every kind).
  *   options      MT_OPT_* bits (below). */
 mt_status mt_set_launch(mt_scene scene, int32_t kind, int32_t threads, int32_t tile, int32_t ctas_per_sm,
                         int32_t priv_bins, uint32_t options);

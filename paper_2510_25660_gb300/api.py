@@ -390,7 +390,9 @@ class Scene:
     def sync(self, stream=None):
         mt_sync(self.h, _stream(stream))
 
-    def set_launch(self, kind, threads=0, tile=0, ctas_per_sm=0, priv_bins=-1, options=0):
+    def set_launch(self, kind, threads=0, tile=0, ctas_per_sm=0, priv_bins=0, options=0):
+        """Launch configuration of `kind`; a call without further arguments restores that of a new scene.
+        priv_bins: -1 = as many bins in shared memory as fit, 0 = none."""
         mt_set_launch(self.h, kind, threads, tile, ctas_per_sm, priv_bins, options)
 
     def set_wavefront_pool(self, max_paths=0):

@@ -58,7 +58,7 @@ def apply(scene, kind, sc, film, spp, depth) -> dict | None:
     if cfg is None and os.path.exists(TABLE):
         cfg = json.load(open(TABLE)).get(key)
     if cfg:
-        scene.set_launch(KINDS[kind], cfg["threads"], cfg["tile"], cfg["ctas_per_sm"], cfg.get("priv", -1),
+        scene.set_launch(KINDS[kind], cfg["threads"], cfg["tile"], cfg["ctas_per_sm"], cfg.get("priv", 0),
                          cfg.get("options", 0))
         if kind != "nlos":
             scene.set_wavefront_pool(pool_paths(cfg.get("paths_per_thread", 0)))

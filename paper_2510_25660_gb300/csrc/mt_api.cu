@@ -674,16 +674,14 @@ static mt_status scene_create_impl(const float *tris, int64_t n, const mt_materi
     D.err = sc->err;
     D.counters = sc->counters;
     al.arena_left = 0;  // later allocations are their own
-    for (int k = 0; k < 4; ++k) sc->cfg[k] = LaunchCfg{256, 0, 0, sc->num_sms, 0, -1, 0};
-    // renders and backward passes add to the film in L2 instead of privatising it: zeroing and writing a
-    // warp's histograms costs more than the few adds of its paths, and the shared memory costs resident
-    // CTAs (97k triangles, 135x241 px, 19 spp: 1150 us against 1628 with all bins that fit; Cornell box
-    // 64x64, 16 spp: 110 against 144 us; backward passes 1291 against 1905 and 176 against 204 us)
-    sc->cfg[MT_LAUNCH_RENDER].priv = sc->cfg[MT_LAUNCH_BACKWARD].priv = 0;
-    sc->cfg[MT_LAUNCH_NLOS].priv = 0;  // 64x64 points, T = 4096, 1024 samples: 1.51 ms against 1.60 privatised
-    // exhaustive NLOS grids: 32 sensors per tile with every splat in global memory (measured 130 ms
-    // against 190 ms at the automatic 6-row tiles with shared-memory histograms)
-    sc->cfg[MT_LAUNCH_NLOS_EXHAUSTIVE] = LaunchCfg{256, 32, 0, sc->num_sms, 0, 0, 0};
+    // The launch defaults, which mt_set_launch with zeros restores.  Nothing is privatised: every contribution is added
+    // to the film in L2.  Renders and backward passes: zeroing and writing a warp's histograms costs more than the few
+    // adds of its paths, and the shared memory costs resident CTAs (97k triangles, 135x241 px, 19 spp: 1150 us against
+    // 1628 with all bins that fit; Cornell box 64x64, 16 spp: 110 against 144 us; backward passes 1291 against 1905
+    // and 176 against 204 us).  Scan points: 64x64, T = 4096, 1024 samples 1.51 ms against 1.60 privatised.
+    // Exhaustive grids: 32 sensors per tile, 130 ms against 190 at the automatic 6-row tiles with shared-memory
+    // histograms (16x16 lasers x 64x64 sensors x 1024 samples, k_nlos).
+    for (int k = 0; k < 4; ++k) sc->cfg[k] = LaunchCfg{256, 0, 0, sc->num_sms, 0, 0, 0};
     return MT_OK;
 }
 
