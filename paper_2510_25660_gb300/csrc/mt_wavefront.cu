@@ -1824,26 +1824,27 @@ mt_status mt_launch_wavefront(const DevScene &s, const WfParams &p0, int num_sms
             }
         }
     }
-    if (known) MT_CUDA_TRY(cudaEventRecord(sync->ev[0], st));
     // one more setup moves the last shading pass's shadow rays and decides whether anything is left
     k_wf_setup<<<1, 1, 0, st>>>(p, p.iter);
     *launches += 1;
+    if (known) MT_CUDA_TRY(cudaEventRecord(sync->ev[0], st));
     MT_TRY(shadow_tail());
     if (timing) {
         MT_CUDA_TRY(cudaStreamSynchronize(st));
         MT_TRY(wf_accumulate(timing, bound));
-    }
-    if (known) {
-        MT_CUDA_TRY(cudaEventSynchronize(sync->ev[0]));
-        return MT_OK;
     }
     if (streamed) {
         MT_CUDA_TRY(cudaEventRecord(sync->ev[bound & 7], st));
         MT_TRY(stream_out_bands(out, sync, sync->ev[bound & 7], true));
     }
     uint32_t done = 0;
-    MT_CUDA_TRY(cudaMemcpyAsync(&done, p.counters + C_DONE, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-    MT_CUDA_TRY(cudaStreamSynchronize(st));
+    if (known) {  // the flag that the setup wrote
+        MT_CUDA_TRY(cudaEventSynchronize(sync->ev[0]));
+        done = *(volatile uint32_t *)sync->done_h == p.done_token ? 1u : 0u;
+    } else {
+        MT_CUDA_TRY(cudaMemcpyAsync(&done, p.counters + C_DONE, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+        MT_CUDA_TRY(cudaStreamSynchronize(st));
+    }
     if (!done) {
         mt::set_error("wavefront render did not drain its queues within the iteration bound");
         return MT_ERR_INTERNAL;
