@@ -652,8 +652,8 @@ def _autograd():
         def backward(ctx, g_film, g_steady):
             scene, T, start, width, spp, seed, max_depth = ctx.args
             albedo, radiance = ctx.saved_tensors
-            if g_film is None and g_steady is None:
-                return (None,) * 11
+            if g_film is None and g_steady is None:  # neither output's gradient is defined: zeros
+                return (torch.zeros_like(albedo), torch.zeros_like(radiance)) + (None,) * 9
             scene.set_params(albedo=albedo.detach().contiguous(), radiance=radiance.detach().contiguous())
             g_film = g_film.contiguous() if g_film is not None else None
             g_steady = g_steady.contiguous() if g_steady is not None else None
