@@ -509,15 +509,9 @@ def render_backward(scene: Scene, T, start, width, spp, seed, max_depth, grad_fi
     import torch
     H, W = grad_film.shape[:2]
     if out is None:
-        n, e = 3 * scene.n_tris, 3 * max(scene.n_em, 1)
-        if n <= 3 << 12:  # small gradients: one cleared buffer (every part starts 16 bytes aligned) instead of three
-            a, b = (n + 3) // 4 * 4, (e + 3) // 4 * 4
-            buf = torch.zeros(a + b + 1, dtype=torch.float32, device="cuda")
-            out = (buf[:n].view(-1, 3), buf[a:a + e].view(-1, 3), buf[a + b:])
-        else:
-            out = (torch.zeros((scene.n_tris, 3), dtype=torch.float32, device="cuda"),
-                   torch.zeros((max(scene.n_em, 1), 3), dtype=torch.float32, device="cuda"),
-                   torch.zeros(1, dtype=torch.float32, device="cuda"))
+        out = tuple(torch.empty(shape, dtype=torch.float32, device="cuda")
+                    for shape in ((scene.n_tris, 3), (max(scene.n_em, 1), 3), (1,)))
+        torch._foreach_zero_(out)  # one kernel clears them all
     galb, grad, gmed = out
     f = Film(grad_film, None, start, width, flags)
     _check_f32([(grad_steady, H * W * 3, "steady-image gradient")])

@@ -1,4 +1,5 @@
-"""TransientRender's backward pass where one output's gradient, or neither, is defined."""
+"""TransientRender's backward pass where one output's gradient, or neither, is defined, and whose memory its gradients
+are."""
 import numpy as np
 import pytest
 
@@ -46,3 +47,12 @@ def test_one_output_used(setup, used):
     both = torch.autograd.grad(film.sum() * (used == "film") + steady.sum() * (used == "steady"), (alb, rad))
     for a, b in zip(only, both):
         assert float(b.abs().max()) > 0 and np.allclose(a.cpu(), b.cpu(), rtol=1e-4, atol=1e-6 * float(b.abs().max()))
+
+
+def test_gradients_own_their_memory(setup):
+    import torch
+    api, s, alb, rad = setup
+    g = api.render_backward(s, 64, 3.5, 0.04, 4, 7, 4, torch.ones((16, 20, 64, 3), device="cuda"))
+    for t in g:
+        assert t._base is None and t.untyped_storage().nbytes() == 4 * t.numel()
+    assert len({t.untyped_storage().data_ptr() for t in g}) == 3
