@@ -641,7 +641,15 @@ static mt_status scene_create_impl(const float *tris, int64_t n, const mt_materi
         D.m_lo = make_float3(med->lo[0], med->lo[1], med->lo[2]);
         D.m_hi = make_float3(med->hi[0], med->hi[1], med->hi[2]);
         D.m_ext = make_float3(med->hi[0] - med->lo[0], med->hi[1] - med->lo[1], med->hi[2] - med->lo[2]);
-        D.m_rext = make_float3(1.0f / D.m_ext.x, 1.0f / D.m_ext.y, 1.0f / D.m_ext.z);
+        // what div_known divides by: an infinite extent (half-open boxes) gives 0 for every finite point, as a / inf
+        // does; so does one whose reciprocal is infinite, in which no point can be told from another
+        float ext[3] = {D.m_ext.x, D.m_ext.y, D.m_ext.z}, rext[3];
+        for (int k = 0; k < 3; ++k) {
+            rext[k] = 1.0f / ext[k];
+            if (!std::isfinite(ext[k]) || !std::isfinite(rext[k])) ext[k] = 1.0f, rext[k] = 0.0f;
+        }
+        D.m_ext = make_float3(ext[0], ext[1], ext[2]);
+        D.m_rext = make_float3(rext[0], rext[1], rext[2]);
         const uint64_t n_cells = (uint64_t)(D.rx + 1) * (D.ry + 1) * (D.rz + 1);
         float4 *cells = nullptr;  // a scene that has no room for them reads the grid
         if (n_cells * 32 <= MT_CELL_BYTES && al.alloc(&cells, 2 * (size_t)n_cells, "density cells") == MT_OK) {

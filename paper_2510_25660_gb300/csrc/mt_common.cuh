@@ -292,7 +292,7 @@ struct DevScene {
     const float *cells;    // the 8 corner densities of every cell, [rz + 1][ry + 1][rx + 1][8] (null: large grids)
     int32_t rx, ry, rz;
     float3 m_lo, m_hi;
-    float3 m_ext, m_rext;  // m_hi - m_lo and its reciprocal, each rounded to nearest
+    float3 m_ext, m_rext;  // m_hi - m_lo and its reciprocal, each rounded to nearest (1 and 0 where either is infinite)
     float m_major;
     const float *m_params; // device [2]: albedo, g
     uint32_t *err;
@@ -306,7 +306,7 @@ __device__ __forceinline__ void raise_err(const DevScene &s, uint32_t bit) { ato
 // ---------------------------------------------------------------------------
 // a / c rounded to nearest, given rc = 1 / c rounded to nearest: a * rc corrected by its exact FMA remainder
 // (Markstein, IBM J. Res. Dev. 34, 1990; Brisebarre, Muller and Raina, IEEE Trans. Computers 53, 2004, for a
-// divisor known in advance).  a and a / c in the normal range.
+// divisor known in advance).  a and a / c in the normal range; 0 for rc = 0.
 __device__ __forceinline__ float div_known(float a, float c, float rc) {
     const float q = a * rc;
     return fmaf(fmaf(-q, c, a), rc, q);
