@@ -588,12 +588,15 @@ static mt_status scene_create_impl(const float *tris, int64_t n, const mt_materi
     MT_TRY(al.alloc(&shrec, (size_t)2 * n, "shading records"));
     k_shading_records<<<g, 256, 0, st>>>(sc->bvh.tris, mats4, tri_unit, (int)n, shrec);
     // Small scenes traced triangle by triangle (trace_flat): in a medium, and where the tree's expected walk (its SAH
-    // cost) is long for so few triangles.  Frames of 128x128 px, 32 spp, depth 6, tree / loop in the persistent form:
-    // in a medium, closed rooms and boxes of 13 to 37 triangles 1022 / 890 to 2325 / 1457 us, random open meshes of 6,
-    // 16, 36, 48, 64 triangles 917 / 741, 1174 / 881, 1436 / 1290, 1476 / 1484, 1560 / 1710, but planes of 2 to 6
-    // triangles 697 / 977 to 1623 / 1828; without one, 20-triangle sphere (SAH cost 12.9) 891 / 471, 37-triangle room
-    // (14.1) 601 / 598, Cornell box (14.3) 611 / 596, 25-triangle room (10.2) 439 / 493, 36 random triangles (5.0) 188 /
-    // 242.  Small frames gain more: Cornell box 64x64, 16 spp 135 / 100.
+    // cost) is long for so few triangles.  Frames of 128x128 px, 32 spp, depth 6, tree / loop in us in the persistent
+    // form.  In a medium: closed rooms and boxes of 13 to 37 triangles 1022 / 890 to 2325 / 1457, random open meshes of
+    // 6, 16, 36, 48, 64 triangles 917 / 741, 1174 / 881, 1436 / 1290, 1476 / 1484, 1560 / 1710, but planes of 2 to 6
+    // triangles 697 / 977 to 1623 / 1828.  Without one (SAH cost in brackets): 20-triangle sphere (12.9) 837 / 464,
+    // Cornell box (14.3) 611 / 583, rooms with random triangles of 32 (12.7), 40 (14.4), 48 (14.2) 600 / 506, 673 / 577,
+    // 749 / 642; below the line rooms with blocks of 25 (10.2) and 37 (12.1) triangles 428 / 459 and 510 / 562, random
+    // open meshes of 8 (2.9), 20 (4.6), 36 (7.0), 48 (8.6) 47 / 53, 78 / 83, 134 / 164, 131 / 172, but rooms with random
+    // triangles of 13 (9.4), 20 (11.6) and 26 (11.5) would gain too: 360 / 346, 508 / 406, 555 / 458; the cost does not
+    // tell them from the blocks.  Small frames gain more: Cornell box 64x64, 16 spp 104 / 79.
     if (n >= 8 && n <= 48 && (med || sc->bvh.sah >= 12.5)) {
         float4 *flat;
         MT_TRY(al.alloc(&flat, (size_t)6 * ((n + 1) / 2), "triangle pairs"));

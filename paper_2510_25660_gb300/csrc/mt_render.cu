@@ -581,8 +581,10 @@ mt_status launch_form(const DevScene &s, const RenderParams &p, const LaunchCfg 
 }
 
 // Small scenes test every triangle in turn when a warp's tile holds enough paths for its lanes to share the work; with
-// fewer lanes the tree's shorter walk is as fast (Cornell box, 64x64 px, 16 spp: 109 -> 79 us; 23x37 px, 1 spp, one
-// path per warp: 37 us in the tree, 39 triangle by triangle).
+// fewer lanes the tree's shorter walk is as fast.  Cornell box, 1 spp, depth 4, frames of 1, 2, 4, 6, 8, 12, 16, 32 paths
+// per warp, tree / loop in us: 51 / 72, 62 / 79, 74 / 83, 82 / 85, 88 / 86, 97 / 91, 102 / 93, 119 / 100; 30-triangle room
+// in a medium 71 / 94, 110 / 133, 151 / 155, 172 / 155, 197 / 164, 235 / 171, 255 / 173, 299 / 173; 20-triangle sphere
+// 67 / 63 to 139 / 83.
 #ifndef MT_FLAT_LANES
 #define MT_FLAT_LANES 8
 #endif
