@@ -289,7 +289,9 @@ __device__ __forceinline__ void em_grad_flush(const WfParams &p, const float *em
 #define MT_FIN_SMEM_TRIS 4096
 #endif
 // Small ones get a copy for each of up to 32 lanes (fin_copies; entry k of copy c at k * copies + c), so that the lanes
-// of a warp do not retry their adds to the same word one after the other.
+// of a warp do not retry their adds to the same word one after the other.  Replay of 128x128 px, 32 spp, depth 8 in
+// rooms of 36, 100, 200, 1000, 4000 triangles, one copy / this rule: 1463 / 1434, 2070 / 2084, 2622 / 2629, 4161 / 4195,
+// 7009 / 7128 us (one copy either way; the rest is the indexing).
 __host__ __device__ __forceinline__ int fin_copies(int n_tris) {
     int c = 32;
     while (c > 1 && 12 * n_tris * c > 48 * 1024) c >>= 1;
